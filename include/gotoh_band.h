@@ -97,9 +97,8 @@ int ga_mlp_loss_grad(const uint16_t *params_bf16, const float *x, const float *t
  * adam_m, adam_v (device float32[6337] each, zero before the first step),
  * and refreshes params_bf16 (round to nearest even).  Bias correction
  * uses step numbers step0+1 .. step0+steps.  losses: device
- * float32[steps] or NULL, the loss of each minibatch.  The steps run as one
- * CUDA graph when `stream` is a created stream not being captured.
- * Synchronises the stream; GA_ERR_ARG also when a batch index is out of
+ * float32[steps] or NULL, the loss of each minibatch.  All steps run in one
+ * kernel launch.  Synchronises the stream; GA_ERR_ARG also when a batch index is out of
  * range.
  */
 int ga_mlp_train(float *master, uint16_t *params_bf16, float *adam_m, float *adam_v, const float *x,

@@ -1,16 +1,13 @@
 // ga_mlp.cu -- training and inference kernels of the band predictor's
 // network and their C ABI (include/gotoh_band.h).  Not part of the paper.
 //
-// A training step is two kernels:
-//   mlp_fwd_bwd_kernel   : thread per batch sample; forward pass with the
-//     bf16 weights (staged once per block in shared memory as float), then
-//     the per-sample backward quantities, written to one scratch row each;
-//   mlp_grad_adam_kernel : thread per parameter; its gradient is the sum
-//     over the batch in sample order (deterministic, no atomics), then the
-//     Adam update of the float32 master value and its bf16 copy.
-// ga_mlp_train records its steps into a CUDA graph and launches that once.
+// Training is one launch for all of its steps (mlp_train_kernel): one cluster
+// of blocks that keeps the parameters on chip and sums every gradient over the
+// batch in sample order (deterministic, no atomics).
+#include <cooperative_groups.h>
+
 #include <cmath>
-#include <cstdio>
+#include <vector>
 
 #include "../../include/gotoh_band.h"
 #include "ga_common.cuh"
@@ -45,128 +42,415 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const uint16_t *__rest
   }
 }
 
-// Thread per batch sample: forward + per-sample backward into scratch rows.
-// idx (nullable) maps batch position -> sample; inv_b = 1 / B.
-__global__ void __launch_bounds__(128) mlp_fwd_bwd_kernel(const uint16_t *__restrict__ wb,
-                                                          const float *__restrict__ x,
-                                                          const float *__restrict__ target,
-                                                          const int32_t *__restrict__ idx, int B,
-                                                          int64_t nsamples, float inv_b,
-                                                          float *__restrict__ scratch,
-                                                          int32_t *__restrict__ status) {
-  extern __shared__ float ws[];
-  const int T = blockDim.x;
-  float *a1 = ws + kParamsPadded + threadIdx.x, *a2 = a1 + kMlpH * T;
-  stage_params(wb, ws);
-  __syncthreads();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int64_t sample = idx ? (int64_t)idx[b] : (int64_t)b;
-  float *row = scratch + (size_t)b * kScratchRow;
-  if (sample < 0 || sample >= nsamples) {  // invalid batch index: zero row, error status
-    for (int c = 0; c < kScratchRow; ++c) row[c] = 0.f;
-    set_status(status, GA_ERR_ARG);
-    return;
-  }
-  const float *xv = x + sample * kMlpIn;
-  for (int i = 0; i < kMlpIn; ++i) row[kSX + i] = xv[i];
-  for (int o = 0; o < kMlpH; ++o) {
-    const float z = unit1(ws, o, xv, 1);
-    a1[o * T] = z;  // pre-activation z1
-    row[kSH1 + o] = fmaxf(z, 0.f);
-  }
-  for (int o = 0; o < kMlpH; ++o) {
-    const float h = fmaxf(unit2(ws, o, a1, T), 0.f);
-    a2[o * T] = h;
-    row[kSH2 + o] = h;
-  }
-  const float y = output(ws, a2, T);
-  const float r = y - target[sample];
-  const float dy = r * inv_b;
-  row[kSDY] = dy;
-  row[kSR] = r;
-  // d2 = dL/dz2 replaces h2 (z2 > 0 exactly where h2 > 0)
-  for (int o = 0; o < kMlpH; ++o) {
-    const float d = a2[o * T] > 0.f ? dy * ws[kOffW3 + o] : 0.f;
-    a2[o * T] = d;
-    row[kSD2 + o] = d;
-  }
-  // d1[i] = relu'(z1[i]) * sum_o d2[o] W2[o][i]
-  for (int i = 0; i < kMlpH; ++i) {
-    float acc = 0.f;
-#pragma unroll 8
-    for (int o = 0; o < kMlpH; ++o) acc = fmaf(a2[o * T], ws[kOffW2 + o * kMlpH + i], acc);
-    row[kSD1 + i] = a1[i * T] > 0.f ? acc : 0.f;
+struct AdamArgs {
+  float lr, beta1, beta2, eps;
+  int update;  // 0: gradient (and loss) only
+};
+
+struct TrainParams {
+  const uint16_t *wb_in;   // bf16 parameters of a gradient-only call (update == 0)
+  float *master;           // float32 parameters, moments and bf16 copy (update != 0)
+  float *adam_m, *adam_v;
+  uint16_t *wb;
+  const float *x;          // [nsamples][32]
+  const float *target;
+  const int32_t *idx;      // [steps][B], or null: samples 0 .. B - 1
+  int64_t nsamples;
+  int32_t steps, B;
+  float inv_b;             // 1 / B
+  const float2 *coef;      // per step: 1 / (1 - beta1^t), 1 / (1 - beta2^t)
+  float *grad_out, *loss_out;
+  int32_t *status;
+  AdamArgs a;
+};
+
+// All Adam steps (or one gradient) in one launch of one cluster of NC blocks.
+//
+// What bounds it: a step is a chain of dependent sums, not work (1.3 MFMA at a
+// batch of 256).  The sums keep the order of the plain loops (a unit's dot
+// product in index order, a parameter's gradient in sample order), so every
+// result is the same float32 value whatever the cluster size; the shortest
+// possible step is then 32 + 64 + 64 + 64 dependent multiply-adds of a sample,
+// 256 of a parameter, and two exchanges.  Two launches per step with a thread
+// per sample and a thread per parameter took 265 us per step at a batch of 256
+// (2 blocks, then 50 blocks of uncoalesced column reads); this takes 14 us, of
+// which about 3.5 us are the forward and backward pass, 2 us the gradients
+// (both at one shared-memory wavefront per cycle), and 7 us the exchanges.
+//
+// Split.  Chunks of 256 samples.  Forward and backward: each block owns SP =
+// 256 / NC samples, a warp four of them: lane l computes units l and l + 32 of
+// its warp's samples, so a layer needs only __syncwarp and every weight read
+// serves four samples.  Gradients: block (p, q) of a 4 x NC/4 grid owns the
+// parameters of 16 units o = 16p.. and 1/(NC/4) of the inputs i of W1 and W2, a
+// 2 x 2 tile per thread, with the master value and both moments in registers
+// for the whole run.  Activations go to the blocks that own the parameters
+// they enter through distributed shared memory, a row of units per store, and
+// new weights the same way to every block.  Two cluster barriers per chunk
+// order the exchanges (activations before the gradients, and everything read
+// before it is overwritten).  The next chunk's inputs are loaded a chunk ahead.
+// The last warp takes the biases, the head and the loss.
+constexpr int kTrChunk = 256;              // samples per chunk
+constexpr int kTrS1 = kMlpIn + 4, kTrS2 = kMlpH + 4;  // padded rows of W1 and W2 in shared memory
+constexpr int kTrW1 = 0, kTrB1 = kTrW1 + kMlpH * kTrS1, kTrW2 = kTrB1 + kMlpH, kTrB2 = kTrW2 + kMlpH * kTrS2,
+              kTrW3 = kTrB2 + kMlpH, kTrB3 = kTrW3 + kMlpH, kTrWeights = kTrB3 + 4;
+
+template <int NC>
+struct TrainShape {
+  static constexpr int Q = NC / 4;                  // blocks along the inputs of a layer
+  static constexpr int I1 = kMlpIn / Q, I2 = kMlpH / Q;  // input columns of W1 and W2 per block
+  static constexpr int SP = kTrChunk / NC;          // samples per block and chunk
+  static constexpr int T = 8 * SP;                  // threads: 4 samples x 32 lanes per warp
+  static constexpr int N2 = 8 * (I2 / 2), N1 = 8 * (I1 / 2);  // threads with a tile of W2, of W1
+  static constexpr int PER = kTrChunk / T;          // staged samples per thread
+  static_assert(N2 + N1 + 32 <= T && PER * I1 == 16, "roles");
+  static constexpr int kAct = 4 * (kMlpIn + 3 * kMlpH);  // floats per warp: x, h1, h2, d2 of 4 samples
+  static constexpr int oD2 = kTrWeights + (T / 32) * kAct, oD1 = oD2 + 16 * kTrChunk,
+                       oH2 = oD1 + 16 * kTrChunk, oH1 = oH2 + 16 * kTrChunk, oX = oH1 + I2 * kTrChunk,
+                       oDY = oX + I1 * kTrChunk, oR = oDY + kTrChunk, kFloats = oR + kTrChunk;
+  static constexpr size_t kSmem = sizeof(float) * kFloats;
+  static_assert(kSmem <= 227 * 1024, "shared memory");
+};
+
+// Position of parameter k in the padded shared-memory copy.
+__device__ __forceinline__ int tr_slot(int k) {
+  if (k < kOffB1) return kTrW1 + (k / kMlpIn) * kTrS1 + k % kMlpIn;
+  if (k < kOffW2) return kTrB1 + (k - kOffB1);
+  if (k < kOffB2) return kTrW2 + ((k - kOffW2) / kMlpH) * kTrS2 + (k - kOffW2) % kMlpH;
+  if (k < kOffW3) return kTrB2 + (k - kOffB2);
+  if (k < kOffB3) return kTrW3 + (k - kOffW3);
+  return kTrB3;
+}
+
+__device__ __forceinline__ float tr_bf16(float w) { return bf16_bits_to_f32(f32_to_bf16_bits(w)); }
+
+struct TrState {  // one parameter's float32 value and moments
+  float w, m, v;
+};
+
+__device__ __forceinline__ void tr_adam(TrState &s, float g, const AdamArgs &a, float2 c) {
+  s.m = fmaf(a.beta1, s.m, (1.f - a.beta1) * g);
+  s.v = fmaf(a.beta2, s.v, (1.f - a.beta2) * g * g);
+  const float mhat = s.m * c.x, vhat = s.v * c.y;
+  s.w = s.w - a.lr * mhat / (sqrtf(vhat) + a.eps);
+}
+
+// Dot products of units l and l + 32 with four samples: z[u][s] += sum_k
+// W[u][k] x[s][k] in index order.
+template <int N, int STRIDE>
+__device__ __forceinline__ void tr_layer(const float *W, const float *x, int l, float (&z)[2][4]) {
+#pragma unroll 4
+  for (int k = 0; k < N; k += 4) {
+    const float4 wa = *reinterpret_cast<const float4 *>(W + l * STRIDE + k);
+    const float4 wc = *reinterpret_cast<const float4 *>(W + (l + 32) * STRIDE + k);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const float4 v = *reinterpret_cast<const float4 *>(x + s * N + k);
+      z[0][s] = fmaf(wa.w, v.w, fmaf(wa.z, v.z, fmaf(wa.y, v.y, fmaf(wa.x, v.x, z[0][s]))));
+      z[1][s] = fmaf(wc.w, v.w, fmaf(wc.z, v.z, fmaf(wc.y, v.y, fmaf(wc.x, v.x, z[1][s]))));
+    }
   }
 }
 
-struct AdamArgs {
-  float lr, beta1, beta2, eps;
-  float c1, c2;  // 1 / (1 - beta1^t), 1 / (1 - beta2^t)
-  int update;    // 0: gradient (and loss) only
-};
+template <int NC>
+__global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __grid_constant__ TrainParams p) {
+  using S = TrainShape<NC>;
+  namespace cg = cooperative_groups;
+  extern __shared__ __align__(16) float tr_smem[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x, l = tid & 31, warp = tid >> 5;
+  const int bp = rank / S::Q, bq = rank % S::Q;
+  float *W = tr_smem;
+  float *xs = tr_smem + kTrWeights + warp * S::kAct, *h1s = xs + 4 * kMlpIn, *h2s = h1s + 4 * kMlpH,
+        *d2s = h2s + 4 * kMlpH;
+  const bool upd = p.a.update != 0;
 
-// Thread per parameter (plus one for the loss): batch sums in sample order.
-__global__ void __launch_bounds__(128) mlp_grad_adam_kernel(const float *__restrict__ scratch, int B,
-                                                            float *__restrict__ master,
-                                                            float *__restrict__ adam_m,
-                                                            float *__restrict__ adam_v,
-                                                            uint16_t *__restrict__ wb,
-                                                            float *__restrict__ grad_out,
-                                                            float *__restrict__ loss_out,
-                                                            const AdamArgs a) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > kMlpParams) return;
-  if (k == kMlpParams) {  // loss
-    if (loss_out) {
-      float s = 0.f;
-      for (int b = 0; b < B; ++b) {
-        const float r = scratch[(size_t)b * kScratchRow + kSR];
-        s = fmaf(r, r, s);
+  for (int k = tid; k < kMlpParams; k += S::T)
+    W[tr_slot(k)] = upd ? tr_bf16(p.master[k]) : bf16_bits_to_f32(p.wb_in[k]);
+
+  // ---- the parameters of this thread --------------------------------------
+  // role 0: 2 x 2 tile of W2, 1: of W1, 2: one parameter or the loss, 3: none
+  int role = 3, par[4] = {-1, -1, -1, -1};  // parameter indices
+  // staged columns (a row per sample): units and inputs, with their row lengths
+  const float *pu = tr_smem, *pv = tr_smem;
+  int su = 16, sv = 16;
+  bool sum_only = false, is_loss = false;
+  if (tid < S::N2) {
+    role = 0;
+    const int o = 2 * (tid / (S::I2 / 2)), i = 2 * (tid % (S::I2 / 2));
+    pu = tr_smem + S::oD2 + o;
+    pv = tr_smem + S::oH1 + i;
+    sv = S::I2;
+    for (int e = 0; e < 4; ++e) par[e] = kOffW2 + (16 * bp + o + (e >> 1)) * kMlpH + S::I2 * bq + i + (e & 1);
+  } else if (tid < S::N2 + S::N1) {
+    role = 1;
+    const int r = tid - S::N2, o = 2 * (r / (S::I1 / 2)), i = 2 * (r % (S::I1 / 2));
+    pu = tr_smem + S::oD1 + o;
+    pv = tr_smem + S::oX + i;
+    sv = S::I1;
+    for (int e = 0; e < 4; ++e) par[e] = kOffW1 + (16 * bp + o + (e >> 1)) * kMlpIn + S::I1 * bq + i + (e & 1);
+  } else if (tid < S::N2 + S::N1 + 32) {
+    const int r = l & 15;
+    if (bq == 0) {
+      role = 2;
+      sum_only = l >= 16;
+      par[0] = (sum_only ? kOffB2 : kOffW3) + 16 * bp + r;
+      pu = tr_smem + (sum_only ? S::oD2 + r : S::oDY);
+      su = sum_only ? 16 : 1;
+      pv = tr_smem + S::oH2 + r;
+    } else if (bq == 1 && l < 16) {
+      role = 2;
+      sum_only = true;
+      par[0] = kOffB1 + 16 * bp + r;
+      pu = tr_smem + S::oD1 + r;
+    } else if (bq == 1 && bp == 0 && l == 16) {
+      role = 2;
+      sum_only = true;
+      par[0] = kOffB3;
+      pu = tr_smem + S::oDY;
+      su = 1;
+    } else if (bq == 1 && bp == 0 && l == 17) {
+      role = 2;
+      is_loss = true;
+      pu = pv = tr_smem + S::oR;
+      su = sv = 1;
+    }
+  }
+  TrState st[4] = {};
+  if (upd)
+    for (int e = 0; e < 4; ++e)
+      if (par[e] >= 0) st[e] = TrState{p.master[par[e]], p.adam_m[par[e]], p.adam_v[par[e]]};
+
+  // ---- inputs of one chunk, loaded a chunk ahead ---------------------------
+  float xv[4], tv = 0.f, xc[S::PER][S::I1];  // own samples (lane = input), target of sample l % 4, staged columns
+  uint32_t ok = 0;                           // bits 0..3: the warp's samples are valid
+  int bad_idx = 0;
+  // the index is only loaded here; it is checked where the inputs are read, so
+  // that nothing waits for it (kNone: no sample at this place)
+  constexpr int64_t kNone = INT64_MIN;
+  auto sample_of = [&](int step, int c0, int b) -> int64_t {
+    if (step >= p.steps || b >= ::min(kTrChunk, p.B - c0)) return kNone;
+    return p.idx ? (int64_t)p.idx[(int64_t)step * p.B + c0 + b] : (int64_t)(c0 + b);
+  };
+  auto own_base = [&](int cb) -> int {  // first sample of this warp in a chunk of cb, or >= cb
+    const int spc = ((cb + NC - 1) / NC + 3) & ~3;
+    return 4 * warp < spc ? rank * spc + 4 * warp : kTrChunk;
+  };
+  int64_t own_s[4], con_s[S::PER];
+  auto read_idx = [&](int step, int c0) {
+    const int sb = own_base(::min(kTrChunk, p.B - c0));
+#pragma unroll
+    for (int s = 0; s < 4; ++s) own_s[s] = sample_of(step, c0, sb + s);
+#pragma unroll
+    for (int j = 0; j < S::PER; ++j) con_s[j] = sample_of(step, c0, tid + j * S::T);
+  };
+  auto read_x = [&]() {
+    ok = 0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      const bool in = own_s[s] >= 0 && own_s[s] < p.nsamples;
+      xv[s] = in ? p.x[own_s[s] * kMlpIn + l] : 0.f;
+      ok |= (in ? 1u : 0u) << s;
+      if ((l & 3) == s) tv = in ? p.target[own_s[s]] : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < S::PER; ++j) {
+      const bool in = con_s[j] >= 0 && con_s[j] < p.nsamples;
+      bad_idx |= !in && con_s[j] != kNone;
+#pragma unroll
+      for (int i = 0; i < S::I1; ++i) xc[j][i] = in ? p.x[con_s[j] * kMlpIn + S::I1 * bq + i] : 0.f;
+    }
+  };
+  read_idx(0, 0);
+  read_x();
+  cluster.sync();  // every block of the cluster runs, its weights are in place
+
+  for (int step = 0; step < p.steps; ++step) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const float2 coef = upd ? p.coef[step] : make_float2(0.f, 0.f);
+    for (int c0 = 0; c0 < p.B; c0 += kTrChunk) {
+      const int cb = ::min(kTrChunk, p.B - c0);
+      const int sb = own_base(cb);
+      // ---- forward and backward of this warp's four samples -----------------
+#pragma unroll
+      for (int j = 0; j < S::PER; ++j)
+#pragma unroll
+        for (int i = 0; i < S::I1; ++i) tr_smem[S::oX + (tid + j * S::T) * S::I1 + i] = xc[j][i];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) xs[s * kMlpIn + l] = xv[s];
+      const float target = tv;
+      const uint32_t valid = ok;
+      const bool last = c0 + kTrChunk >= p.B;
+      read_idx(last ? step + 1 : step, last ? 0 : c0 + kTrChunk);
+      __syncwarp();
+      if (sb < cb) {
+        float z[2][4], h1[2][4], h2[2][4], d2[2][4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          z[0][s] = W[kTrB1 + l];
+          z[1][s] = W[kTrB1 + l + 32];
+        }
+        tr_layer<kMlpIn, kTrS1>(W + kTrW1, xs, l, z);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int s = 0; s < 4; ++s) h1s[s * kMlpH + l + 32 * u] = h1[u][s] = fmaxf(z[u][s], 0.f);
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          z[0][s] = W[kTrB2 + l];
+          z[1][s] = W[kTrB2 + l + 32];
+        }
+        tr_layer<kMlpH, kTrS2>(W + kTrW2, h1s, l, z);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int s = 0; s < 4; ++s) h2s[s * kMlpH + l + 32 * u] = h2[u][s] = fmaxf(z[u][s], 0.f);
+        __syncwarp();
+        float y = W[kTrB3];
+        const float *hv = h2s + (l & 3) * kMlpH;
+#pragma unroll 4
+        for (int o = 0; o < kMlpH; o += 4) {
+          const float4 w = *reinterpret_cast<const float4 *>(W + kTrW3 + o);
+          const float4 v = *reinterpret_cast<const float4 *>(hv + o);
+          y = fmaf(w.w, v.w, fmaf(w.z, v.z, fmaf(w.y, v.y, fmaf(w.x, v.x, y))));
+        }
+        const bool mine = (valid >> (l & 3)) & 1u;
+        const float r = mine ? y - target : 0.f, dy = mine ? r * p.inv_b : 0.f;
+        float dys[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) dys[s] = __shfl_sync(0xffffffffu, dy, s);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int s = 0; s < 4; ++s)
+            d2s[s * kMlpH + l + 32 * u] = d2[u][s] = h2[u][s] > 0.f ? dys[s] * W[kTrW3 + l + 32 * u] : 0.f;
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < 4; ++s) z[0][s] = z[1][s] = 0.f;
+#pragma unroll 2
+        for (int o = 0; o < kMlpH; o += 4) {
+          float wa[4], wc[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            wa[j] = W[kTrW2 + (o + j) * kTrS2 + l];
+            wc[j] = W[kTrW2 + (o + j) * kTrS2 + l + 32];
+          }
+#pragma unroll
+          for (int s = 0; s < 4; ++s) {
+            const float4 d = *reinterpret_cast<const float4 *>(d2s + s * kMlpH + o);
+            z[0][s] = fmaf(d.w, wa[3], fmaf(d.z, wa[2], fmaf(d.y, wa[1], fmaf(d.x, wa[0], z[0][s]))));
+            z[1][s] = fmaf(d.w, wc[3], fmaf(d.z, wc[2], fmaf(d.y, wc[1], fmaf(d.x, wc[0], z[1][s]))));
+          }
+        }
+        // ---- to the blocks that own the parameters ---------------------------
+        auto put = [&](int dst, int at, float v) { *cluster.map_shared_rank(tr_smem + at, dst) = v; };
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          const int b = sb + s;
+          const bool keep = (valid >> s) & 1u;  // an invalid sample adds nothing
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const int unit = l + 32 * u, ub = unit / 16 * S::Q, uo = b * 16 + unit % 16;
+            const float e1 = keep ? h1[u][s] : 0.f, e2 = keep ? d2[u][s] : 0.f;
+            const float e3 = keep && h1[u][s] > 0.f ? z[u][s] : 0.f;
+#pragma unroll
+            for (int r4 = 0; r4 < 4; ++r4)
+              put(r4 * S::Q + unit / S::I2, S::oH1 + b * S::I2 + unit % S::I2, e1);
+#pragma unroll
+            for (int q = 0; q < S::Q; ++q) {
+              put(ub + q, S::oD2 + uo, e2);
+              put(ub + q, S::oD1 + uo, e3);
+            }
+            put(ub, S::oH2 + uo, keep ? h2[u][s] : 0.f);
+          }
+        }
+        if (l < 20) {  // the head's error signal to the blocks that own the head, the error to the loss
+          const int s = l & 3, d = l >> 2;
+          put(d < 4 ? d * S::Q : 1, S::oDY + sb + s, dy);
+          if (d == 4) put(1, S::oR + sb + s, r);
+        }
       }
-      *loss_out = 0.5f * s / (float)B;
+      read_x();  // the next chunk's inputs arrive while the gradients run
+      cluster.sync();
+      // ---- gradients, in sample order ---------------------------------------
+      if (role < 2) {
+        // eight samples are loaded while the eight before them are summed
+        float2 a[8], c[8];
+        auto load8 = [&](int b) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            a[j] = *reinterpret_cast<const float2 *>(pu + (b + j) * 16);
+            c[j] = *reinterpret_cast<const float2 *>(pv + (b + j) * sv);
+          }
+        };
+        load8(0);
+        int b = 0;
+        for (; b + 8 <= cb; b += 8) {
+          float2 a0[8], c0v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            a0[j] = a[j];
+            c0v[j] = c[j];
+          }
+          load8(::min(b + 8, kTrChunk - 8));
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            acc[0] = fmaf(a0[j].x, c0v[j].x, acc[0]);
+            acc[1] = fmaf(a0[j].x, c0v[j].y, acc[1]);
+            acc[2] = fmaf(a0[j].y, c0v[j].x, acc[2]);
+            acc[3] = fmaf(a0[j].y, c0v[j].y, acc[3]);
+          }
+        }
+        for (; b < cb; ++b) {
+          const float2 e = *reinterpret_cast<const float2 *>(pu + b * 16);
+          const float2 f = *reinterpret_cast<const float2 *>(pv + b * sv);
+          acc[0] = fmaf(e.x, f.x, acc[0]);
+          acc[1] = fmaf(e.x, f.y, acc[1]);
+          acc[2] = fmaf(e.y, f.x, acc[2]);
+          acc[3] = fmaf(e.y, f.y, acc[3]);
+        }
+      } else if (role == 2) {
+#pragma unroll 8
+        for (int b = 0; b < cb; ++b) acc[0] = fmaf(pu[b * su], sum_only ? 1.f : pv[b * sv], acc[0]);
+      }
+      if (last) {
+        if (is_loss && p.loss_out) p.loss_out[step] = 0.5f * acc[0] / (float)p.B;
+        if (p.grad_out)
+          for (int e = 0; e < 4; ++e)
+            if (par[e] >= 0) p.grad_out[par[e]] = acc[e];
+        if (upd && role < 2) {
+          float n[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            tr_adam(st[e], acc[e], p.a, coef);
+            n[e] = tr_bf16(st[e].w);
+          }
+          const int at0 = tr_slot(par[0]), at1 = tr_slot(par[2]);
+#pragma unroll
+          for (int r = 0; r < NC; ++r) {
+            *reinterpret_cast<float2 *>(cluster.map_shared_rank(W + at0, r)) = make_float2(n[0], n[1]);
+            *reinterpret_cast<float2 *>(cluster.map_shared_rank(W + at1, r)) = make_float2(n[2], n[3]);
+          }
+        } else if (upd && role == 2 && !is_loss) {
+          tr_adam(st[0], acc[0], p.a, coef);
+          const float n = tr_bf16(st[0].w);
+          const int at = tr_slot(par[0]);
+#pragma unroll
+          for (int r = 0; r < NC; ++r) *cluster.map_shared_rank(W + at, r) = n;
+        }
+      }
+      cluster.sync();
     }
-    return;
   }
-  int ua, ub;  // scratch columns multiplied: g = sum_b row[ua] * (ub < 0 ? 1 : row[ub])
-  if (k < kOffB1) {
-    ua = kSD1 + k / kMlpIn;
-    ub = kSX + k % kMlpIn;
-  } else if (k < kOffW2) {
-    ua = kSD1 + (k - kOffB1);
-    ub = -1;
-  } else if (k < kOffB2) {
-    ua = kSD2 + (k - kOffW2) / kMlpH;
-    ub = kSH1 + (k - kOffW2) % kMlpH;
-  } else if (k < kOffW3) {
-    ua = kSD2 + (k - kOffB2);
-    ub = -1;
-  } else if (k < kOffB3) {
-    ua = kSDY;
-    ub = kSH2 + (k - kOffW3);
-  } else {
-    ua = kSDY;
-    ub = -1;
-  }
-  float g = 0.f;
-  if (ub >= 0) {
-    for (int b = 0; b < B; ++b) {
-      const float *row = scratch + (size_t)b * kScratchRow;
-      g = fmaf(row[ua], row[ub], g);
-    }
-  } else {
-    for (int b = 0; b < B; ++b) g += scratch[(size_t)b * kScratchRow + ua];
-  }
-  if (grad_out) grad_out[k] = g;
-  if (!a.update) return;
-  const float mk = fmaf(a.beta1, adam_m[k], (1.f - a.beta1) * g);
-  const float vk = fmaf(a.beta2, adam_v[k], (1.f - a.beta2) * g * g);
-  adam_m[k] = mk;
-  adam_v[k] = vk;
-  const float mhat = mk * a.c1, vhat = vk * a.c2;
-  const float w = master[k] - a.lr * mhat / (sqrtf(vhat) + a.eps);
-  master[k] = w;
-  wb[k] = f32_to_bf16_bits(w);
+  if (bad_idx && p.status) set_status(p.status, GA_ERR_ARG);
+  if (upd)
+    for (int e = 0; e < 4; ++e)
+      if (par[e] >= 0) {
+        p.master[par[e]] = st[e].w;
+        p.adam_m[par[e]] = st[e].m;
+        p.adam_v[par[e]] = st[e].v;
+        p.wb[par[e]] = f32_to_bf16_bits(st[e].w);
+      }
 }
 
 // Cast of a float32 parameter vector to bf16 (round to nearest even).
@@ -185,8 +469,6 @@ int mlp_smem_ok() {  // per call: the attribute belongs to the current device
   int ok = 0;
   {
     ok = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)kParamSmem) == cudaSuccess &&
-         cudaFuncSetAttribute(mlp_fwd_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)kParamSmem) == cudaSuccess;
   }
   return ok;
@@ -203,17 +485,48 @@ struct Scratch {
   }
 };
 
-// One training (or gradient-only) step on the batch idx[0..B) (idx null:
-// samples 0..B-1).
-cudaError_t enqueue_step(const uint16_t *wb, const float *x, const float *target, int64_t nsamples,
-                         const int32_t *idx, int B, float *scratch, int32_t *status, float *master,
-                         float *am, float *av, uint16_t *wb_out, float *grad, float *loss,
-                         const AdamArgs &a, cudaStream_t s) {
-  mlp_fwd_bwd_kernel<<<(B + kMlpThreads - 1) / kMlpThreads, kMlpThreads, kParamSmem, s>>>(
-      wb, x, target, idx, B, nsamples, 1.0f / (float)B, scratch, status);
-  mlp_grad_adam_kernel<<<(kMlpParams + 1 + kMlpThreads - 1) / kMlpThreads, kMlpThreads, 0, s>>>(
-      scratch, B, master, am, av, wb_out, grad, loss, a);
-  return cudaGetLastError();
+template <int NC>
+cudaError_t launch_train(const TrainParams &p, cudaStream_t s, bool only_if_it_fits, bool *launched) {
+  using S = TrainShape<NC>;
+  *launched = false;
+  cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+  if (e == cudaSuccess && NC > 8)
+    e = cudaFuncSetAttribute(mlp_train_kernel<NC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(NC);
+  cfg.blockDim = dim3(S::T);
+  cfg.dynamicSmemBytes = S::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = NC;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (only_if_it_fits) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, mlp_train_kernel<NC>, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      return cudaSuccess;
+    }
+  }
+  *launched = true;
+  return cudaLaunchKernelEx(&cfg, mlp_train_kernel<NC>, p);
+}
+
+// Cluster size: 8 blocks below 96 samples a step, where a chunk keeps few warps
+// busy and a smaller cluster exchanges faster (GB300, us per step, 16 / 8
+// blocks: 8.5 / 7.8 at 16 samples, 8.9 / 8.8 at 64, 10.2 / 10.8 at 128, 13.8 /
+// 16.2 at 256, 46 / 58 at 1024); 8 is also the portable size where a device
+// places no cluster of 16.  The results are the same.
+cudaError_t enqueue_train(const TrainParams &p, cudaStream_t s) {
+  bool launched = false;
+  if (p.B >= 96) {
+    const cudaError_t e = launch_train<16>(p, s, true, &launched);
+    if (e != cudaSuccess || launched) return e;
+  }
+  return launch_train<8>(p, s, false, &launched);
 }
 
 }  // namespace
@@ -240,15 +553,17 @@ int ga_mlp_forward(const uint16_t *params_bf16, const float *x, int64_t n, float
 int ga_mlp_loss_grad(const uint16_t *params_bf16, const float *x, const float *target, int32_t n,
                      float *grad, float *loss, void *stream) {
   if (n <= 0 || !params_bf16 || !x || !target || !grad) return GA_ERR_ARG;
-  if (!mlp_smem_ok()) return GA_ERR_CUDA;
-  cudaStream_t s = (cudaStream_t)stream;
-  Scratch sc(s, sizeof(float) * (size_t)n * kScratchRow + 256);
-  if (!sc.p) return GA_ERR_OOM;
-  AdamArgs a{};
-  a.update = 0;
-  const cudaError_t e = enqueue_step(params_bf16, x, target, n, nullptr, n, (float *)sc.p, nullptr,
-                                     nullptr, nullptr, nullptr, nullptr, grad, loss, a, s);
-  return e == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+  TrainParams p{};
+  p.wb_in = params_bf16;
+  p.x = x;
+  p.target = target;
+  p.nsamples = n;
+  p.steps = 1;
+  p.B = n;
+  p.inv_b = 1.0f / (float)n;
+  p.grad_out = grad;
+  p.loss_out = loss;
+  return enqueue_train(p, (cudaStream_t)stream) == cudaSuccess ? GA_OK : GA_ERR_CUDA;
 }
 
 int ga_mlp_train(float *master, uint16_t *params_bf16, float *adam_m, float *adam_v, const float *x,
@@ -260,59 +575,37 @@ int ga_mlp_train(float *master, uint16_t *params_bf16, float *adam_m, float *ada
   if (!(lr > 0.f) || !(beta1 >= 0.f && beta1 < 1.f) || !(beta2 >= 0.f && beta2 < 1.f) || !(eps >= 0.f))
     return GA_ERR_ARG;
   if (steps == 0) return GA_OK;
-  if (!mlp_smem_ok()) return GA_ERR_CUDA;
   cudaStream_t s = (cudaStream_t)stream;
-  Scratch sc(s, sizeof(float) * (size_t)batch * kScratchRow + 256);
-  if (!sc.p) return GA_ERR_OOM;
-  float *scratch = (float *)sc.p;
-  Scratch st(s, 256);
+  Scratch st(s, 256 + sizeof(float2) * (size_t)steps);
   if (!st.p) return GA_ERR_OOM;
   int32_t *status = (int32_t *)st.p;
-  if (cudaMemsetAsync(status, 0, sizeof(int32_t), s) != cudaSuccess) return GA_ERR_CUDA;
-  // bf16 copy of the current master weights
-  mlp_cast_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(master, params_bf16, kMlpParams);
-
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return GA_ERR_CUDA;
-  const bool graph = s != nullptr && cap == cudaStreamCaptureStatusNone && steps > 1;
-  auto enqueue_all = [&]() -> cudaError_t {
-    for (int k = 0; k < steps; ++k) {
-      const double t = (double)step0 + k + 1;
-      AdamArgs a{};
-      a.lr = lr;
-      a.beta1 = beta1;
-      a.beta2 = beta2;
-      a.eps = eps;
-      a.c1 = (float)(1.0 / (1.0 - std::pow((double)beta1, t)));
-      a.c2 = (float)(1.0 / (1.0 - std::pow((double)beta2, t)));
-      a.update = 1;
-      const cudaError_t e = enqueue_step(params_bf16, x, target, nsamples, batch_idx + (size_t)k * batch,
-                                         batch, scratch, status, master, adam_m, adam_v, params_bf16,
-                                         nullptr, losses ? losses + k : nullptr, a, s);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  };
-  if (graph) {
-    cudaGraph_t g = nullptr;
-    cudaGraphExec_t ge = nullptr;
-    if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return GA_ERR_CUDA;
-    const cudaError_t e1 = enqueue_all();
-    const cudaError_t e2 = cudaStreamEndCapture(s, &g);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || !g) {
-      if (g) cudaGraphDestroy(g);
-      return GA_ERR_CUDA;
-    }
-    const cudaError_t e3 = cudaGraphInstantiate(&ge, g, 0);
-    cudaGraphDestroy(g);
-    if (e3 != cudaSuccess) return GA_ERR_CUDA;
-    const cudaError_t e4 = cudaGraphLaunch(ge, s);
-    const cudaError_t e5 = cudaStreamSynchronize(s);
-    cudaGraphExecDestroy(ge);
-    if (e4 != cudaSuccess || e5 != cudaSuccess) return GA_ERR_CUDA;
-  } else {
-    if (enqueue_all() != cudaSuccess) return GA_ERR_CUDA;
+  float2 *coef = (float2 *)((char *)st.p + 256);
+  std::vector<float2> h_coef((size_t)steps);  // bias corrections, in double on the host
+  for (int k = 0; k < steps; ++k) {
+    const double t = (double)step0 + k + 1;
+    h_coef[k] = make_float2((float)(1.0 / (1.0 - std::pow((double)beta1, t))),
+                            (float)(1.0 / (1.0 - std::pow((double)beta2, t))));
   }
+  if (cudaMemsetAsync(status, 0, sizeof(int32_t), s) != cudaSuccess ||
+      cudaMemcpyAsync(coef, h_coef.data(), sizeof(float2) * h_coef.size(), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return GA_ERR_CUDA;
+  TrainParams p{};
+  p.master = master;
+  p.adam_m = adam_m;
+  p.adam_v = adam_v;
+  p.wb = params_bf16;
+  p.x = x;
+  p.target = target;
+  p.idx = batch_idx;
+  p.nsamples = nsamples;
+  p.steps = steps;
+  p.B = batch;
+  p.inv_b = 1.0f / (float)batch;
+  p.coef = coef;
+  p.loss_out = losses;
+  p.status = status;
+  p.a = AdamArgs{lr, beta1, beta2, eps, 1};
+  if (enqueue_train(p, s) != cudaSuccess) return GA_ERR_CUDA;
   int32_t h = 0;
   if (cudaMemcpyAsync(&h, status, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)

@@ -19,12 +19,7 @@ constexpr int kOffW1 = 0, kOffB1 = kOffW1 + kMlpH * kMlpIn, kOffW2 = kOffB1 + kM
               kOffB2 = kOffW2 + kMlpH * kMlpH, kOffW3 = kOffB2 + kMlpH, kOffB3 = kOffW3 + kMlpH;
 constexpr int kMlpParams = kOffB3 + 1;  // 6337
 constexpr int kMlpParamsPadded = (kMlpParams + 3) & ~3;
-// Per-sample scratch row: x, h1, d1 (dL/dz1), h2, d2 (dL/dz2), dy, r.
-constexpr int kSX = 0, kSH1 = kSX + kMlpIn, kSD1 = kSH1 + kMlpH, kSH2 = kSD1 + kMlpH,
-              kSD2 = kSH2 + kMlpH, kSDY = kSD2 + kMlpH, kSR = kSDY + 1;
-constexpr int kScratchRow = 292;  // >= kSR + 1, multiple of 4
 static_assert(kMlpParams == 6337, "parameter layout");
-static_assert(kScratchRow >= kSR + 1, "scratch row");
 
 __device__ __forceinline__ float bf16_bits_to_f32(uint16_t b) {
   return __uint_as_float((uint32_t)b << 16);

@@ -1,0 +1,64 @@
+"""GPU: the one-launch training kernel at the edges of its chunks (256 samples),
+of its warps (4 samples) and of the rule that picks its cluster size (96)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import mlp as omlp
+from synth.band import mlp_init
+
+import paper_2205_07610_gb300 as ga
+
+pytestmark = pytest.mark.gpu
+
+SIZES = (1, 3, 4, 31, 95, 96, 97, 255, 256, 257, 600)
+
+
+def _problem(n, seed):
+    rng = np.random.default_rng(seed)
+    x = rng.uniform(0, 1, size=(n, 32)).astype(np.float32)
+    t = rng.uniform(0, 12, size=n).astype(np.float32)
+    return mlp_init(seed), x, t
+
+
+@pytest.mark.parametrize("n", SIZES)
+def test_gradient_parity(n):
+    p, x, t = _problem(n, 40 + n)
+    wb = ga.mlp_cast(torch.from_numpy(p).cuda())
+    p64 = (wb.cpu().numpy().view(np.uint16).astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+    loss, g = ga.mlp_loss_grad(wb, torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda())
+    L, gref = omlp.loss_grad(p64, x.astype(np.float64), t.astype(np.float64))
+    # float32 sums of n terms: (n + 160) roundings of 2^-24 of the largest terms
+    tol = (n + 160) * 2.0 ** -24
+    assert abs(float(loss.item()) - L) <= 4 * tol * max(1.0, L)
+    scale = np.abs(t).max() * max(1.0, np.abs(p64).max()) * 8
+    assert np.max(np.abs(g.cpu().numpy() - gref)) <= 4 * tol * scale + 1e-6
+
+
+@pytest.mark.parametrize("n", SIZES)
+def test_steps_in_one_launch_equal_single_steps(n):
+    p, x, t = _problem(300, 70 + n)
+    X, T = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    idx = torch.from_numpy(np.random.default_rng(n).integers(0, 300, size=(3, n)).astype(np.int32)).cuda()
+    runs = []
+    for cut in ([3], [1, 1, 1]):
+        master = torch.from_numpy(p.copy()).cuda()
+        am, av = torch.zeros_like(master), torch.zeros_like(master)
+        wb = ga.mlp_cast(master)
+        losses, k = [], 0
+        for s in cut:
+            losses.append(ga.mlp_train(master, wb, am, av, X, T, idx[k:k + s].contiguous(), step0=k, lr=1e-3))
+            k += s
+        runs.append([a.cpu().numpy() for a in (master, am, av, wb, torch.cat(losses))])
+    for a, b in zip(*runs):
+        np.testing.assert_array_equal(a, b)
+    np.testing.assert_array_equal(runs[0][3].view(np.uint16), omlp.bf16_bits(runs[0][0]))
+
+
+def test_negative_batch_index_is_refused():
+    p, x, t = _problem(10, 3)
+    master = torch.from_numpy(p).cuda()
+    idx = torch.tensor([[0, 5, -1]], dtype=torch.int32, device="cuda")
+    with pytest.raises(ga.GotohError):
+        ga.mlp_train(master, ga.mlp_cast(master), torch.zeros_like(master), torch.zeros_like(master),
+                     torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda(), idx)
