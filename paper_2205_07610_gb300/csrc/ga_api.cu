@@ -2,6 +2,7 @@
 // planning (encode, classify, length sort) and kernel dispatch.
 #include <algorithm>
 #include <memory>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -14,8 +15,10 @@
 #include "ga_pool.h"
 #include "ga_prot.cuh"
 #include "ga_serve_host.h"
+#include "ga_kx.h"
 #include "ga_launch.h"
 #include "ga_prep.cuh"
+#include "ga_strip_tasks.cuh"
 
 namespace ga {
 
@@ -156,6 +159,15 @@ struct Alloc {
     ptrs.push_back(p);
     return (T *)p;
   }
+  // As get, for memory that the call can do without: null when there is none.
+  template <class T>
+  T *try_get(size_t n) {
+    const bool was = failed;
+    T *p = get<T>(n);
+    if (!p) cudaGetLastError();
+    failed = was;
+    return p;
+  }
   ~Alloc() {
     for (void *p : ptrs) cudaFreeAsync(p, s);
   }
@@ -178,6 +190,7 @@ void *pinned_scratch() {
 struct Small {
   int32_t status;
   int32_t rmax_long;
+  LongSums long_sums;
   unsigned long long cells;
   int32_t rerun_total;
   int32_t pad0;
@@ -194,6 +207,7 @@ struct Small {
 struct Readback {
   int32_t status;
   int32_t rmax_long;
+  LongSums long_sums;
   unsigned long long cells;
   int32_t rerun_total;
   int32_t pad0;
@@ -424,6 +438,8 @@ struct ChunkPlan {
   int64_t long_stride = 0;
   size_t long_smem = 0;
   int2 *long_bnd = nullptr;
+  int kx_tile = -1;  // >= 0: the long class runs as strip tasks (ga_strip.cuh)
+  KXParams kx{};
 };
 
 // Plan and sort kernels of one plan, on the call's stream.
@@ -433,7 +449,8 @@ int plan_enqueue(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   if (cudaMemsetAsync(&p.sm->counters, 0, sizeof(p.sm->counters) + sizeof(p.sm->rerun_range), c.s) !=
       cudaSuccess)
     return GA_ERR_CUDA;
-  if (cudaMemsetAsync(&p.sm->rmax_long, 0, sizeof(int32_t), c.s) != cudaSuccess) return GA_ERR_CUDA;
+  if (cudaMemsetAsync(&p.sm->rmax_long, 0, offsetof(Small, cells) - offsetof(Small, rmax_long), c.s) != cudaSuccess)
+    return GA_ERR_CUDA;
 
   PlanParams pp{};
   pp.q_off = Q.off;
@@ -457,6 +474,7 @@ int plan_enqueue(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   pp.status = &c.small->status;
   pp.cells = &c.small->cells;
   pp.rmax_long = &p.sm->rmax_long;
+  pp.long_sums = &p.sm->long_sums;
   const unsigned tb = 256;
   const unsigned nb = (unsigned)((p.npairs + tb - 1) / tb);
   plan_kernel<<<nb, tb, 0, c.s>>>(pp);
@@ -491,9 +509,72 @@ int plan_bin_count(const ChunkPlan &p, int cls, int bin) {
   return p.r.ranges[2 * key + 1] - p.r.ranges[2 * key];
 }
 
+// Strip launch of a plan's long class: the task list and the zeroed edge words,
+// one buffer of (shorter sequence + 1) words per pair.  Left to the kernels that
+// run a pair on one warp where the relative int16 cells of the scoring are not
+// exact, a pair has too many strips, or the edges would take more than 4 GB.
+int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
+  p.kx_tile = -1;
+  if (std::max(c.sc.smax, 0) + c.sc.alpha > kKxMaxStep) return GA_OK;
+  const LongSums &ls = p.r.long_sums;
+  int64_t strips[kKxWidths];
+  for (int w = 0; w < kKxWidths; ++w) strips[w] = ls.strips[w];
+  const int tile = kx_choose(p.mode, !c.dna, p.r.rmax_long, strips, c.nsm);
+  const int64_t W = 64 * kKxTileK[tile], ntasks = strips[kKxTileK[tile] / 4 - 1];
+  if (p.r.rmax_long > W * kKxMaxStrips || ntasks > (1 << 30) || ls.rows > (4ull << 30) / 8) return GA_OK;
+  const int64_t cnt = p.long_cnt;
+  const size_t head = sizeof(KXPairState) * (size_t)cnt + 16, bytes = head + 8 * (size_t)ls.rows;
+  char *zero = c.al.try_get<char>(bytes);
+  int2 *tasks = zero ? c.al.try_get<int2>((size_t)ntasks) : nullptr;
+  int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)cnt) : nullptr;
+  if (!edge_off) return GA_OK;
+  KXParams &k = p.kx;
+  k = KXParams{};
+  k.q_codes = Q.codes;
+  k.t_codes = T.codes;
+  k.q_off = Q.off;
+  k.t_off = T.off;
+  k.sorted = p.sorted;
+  k.range = &p.sm->ranges[2 * (kClassLong * kBins)];
+  k.tasks = tasks;
+  k.ntasks = (int32_t)ntasks;
+  k.state = reinterpret_cast<KXPairState *>(zero);
+  k.counter = reinterpret_cast<int32_t *>(zero + sizeof(KXPairState) * (size_t)cnt);
+  k.edge_off = edge_off;
+  k.edges = reinterpret_cast<unsigned long long *>(zero + head);
+  k.scores = p.scores;
+  k.status = &c.small->status;
+  k.nt = p.nt;
+  k.q0 = p.q0;
+  std::memcpy(k.tables, c.sc.tables, sizeof(k.tables));
+  std::memcpy(k.sigma, c.sc.mat, sizeof(k.sigma));
+  k.A = c.sc.A;
+  k.alpha = c.sc.alpha;
+  k.beta = c.sc.beta;
+  int occ = 0;
+  if (launch_kx(p.mode, tile, k, 0, c.s, &occ) != cudaSuccess) return GA_ERR_CUDA;
+  p.long_grid = (int)std::min<int64_t>((ntasks + kKxWarps - 1) / kKxWarps, (int64_t)c.nsm * std::max(occ, 1));
+  KXTaskParams kt{};
+  kt.q_off = Q.off;
+  kt.t_off = T.off;
+  kt.sorted = k.sorted;
+  kt.range = k.range;
+  kt.nt = p.nt;
+  kt.q0 = p.q0;
+  kt.W = (int32_t)W;
+  kt.tasks = tasks;
+  kt.edge_off = edge_off;
+  if (cudaMemsetAsync(zero, 0, bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
+  kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
+  ++c.launches;
+  if (cudaGetLastError() != cudaSuccess) return GA_ERR_CUDA;
+  p.kx_tile = tile;
+  return GA_OK;
+}
+
 // Launch count, long-class grid and edge buffer of a read-back plan.  The
 // buffer is allocated here, before the fork: the side streams start after it.
-int launch_prepare(Call &c, ChunkPlan &p) {
+int launch_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   p.nlaunch = 0;
   p.counter = 0;
   if (p.npairs == 0) return GA_OK;
@@ -504,6 +585,8 @@ int launch_prepare(Call &c, ChunkPlan &p) {
   const bool profile = !c.dna;
   p.long_smem = profile ? (size_t)kKbWarps * (size_t)(c.sc.A + 1) * (32 * kKbK) : 0;
   if (p.long_cnt > 0) {
+    if (int rc = kx_prepare(c, Q, T, p)) return rc;
+    if (p.kx_tile >= 0) return GA_OK;
     int occ = 0;
     if (long_packed(c.sc, c.dna))
       occ = p.mode == GA_LOCAL ? blocks_per_sm_kw_local()
@@ -610,6 +693,13 @@ int launch_bin(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p, int cl
 // Long pairs (and every pair of an alphabet of more than 4 symbols) of a plan.
 int launch_long(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p, DpFork &fk) {
   if (p.npairs == 0 || p.long_cnt <= 0) return GA_OK;
+  if (p.kx_tile >= 0) {
+    c.pairs16 += p.long_cnt;
+    const cudaStream_t ls = fk.launch_begin();
+    const cudaError_t e = launch_kx(p.mode, p.kx_tile, p.kx, p.long_grid, ls);
+    fk.launch_end();
+    return e == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+  }
   const bool profile = !c.dna;
   const bool packed = long_packed(c.sc, c.dna);
   (packed ? c.pairs16 : c.pairs32) += p.long_cnt;
@@ -701,7 +791,7 @@ int run_plans(Call &c, const SetView &Q, const SetView &T, ChunkPlan *ps, int n)
     if ((rc = plan_enqueue(c, Q, T, ps[k]))) return rc;
   if ((rc = plan_readback(c, ps, n))) return rc;
   for (int k = 0; k < n; ++k)
-    if ((rc = launch_prepare(c, ps[k]))) return rc;
+    if ((rc = launch_prepare(c, Q, T, ps[k]))) return rc;
   if ((rc = launch_plans(c, Q, T, ps, n))) return rc;
   for (int k = 0; k < n; ++k)
     if ((rc = rerun_enqueue(c, Q, T, ps[k]))) return rc;
@@ -813,6 +903,59 @@ int batch_modes_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t
   }
   if ((rc = run_plans(c, Q, T, ps, nmodes))) return rc;
   return finish(c, stats, ev.e0, ev.e1, npairs * nmodes);
+}
+
+// One pair of at least one residue each on strip tasks, without planning.
+int kx_align_pair(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, const Scoring &sc, int mode,
+                  int32_t *score, cudaStream_t s, ga_stats *stats) {
+  Call c(s);
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return GA_ERR_CUDA;
+  const int64_t R = std::min(m, n), C = std::max(m, n);
+  int64_t strips[kKxWidths];
+  for (int w = 0; w < kKxWidths; ++w) strips[w] = (C + kx_width(w) - 1) / kx_width(w);
+  const int tile = kx_choose(mode, sc.A > 4, R, strips, c.nsm);
+  const int64_t ns = strips[kKxTileK[tile] / 4 - 1];
+  const size_t head = sizeof(KXPairState) + 16, bytes = head + (ns > 1 ? 8 * (size_t)(R + 1) : 0);
+  Events ev(stats != nullptr, s);
+  char *zero = c.al.get<char>(bytes);
+  if (!zero) return GA_ERR_OOM;
+  KXParams k{};
+  k.q_codes = q;
+  k.t_codes = t;
+  k.m = (int32_t)m;
+  k.n = (int32_t)n;
+  k.ntasks = (int32_t)ns;
+  k.state = reinterpret_cast<KXPairState *>(zero);
+  k.counter = reinterpret_cast<int32_t *>(zero + sizeof(KXPairState));
+  k.edges = reinterpret_cast<unsigned long long *>(zero + head);
+  k.scores = score;
+  k.status = k.counter + 1;
+  std::memcpy(k.tables, sc.tables, sizeof(k.tables));
+  std::memcpy(k.sigma, sc.mat, sizeof(k.sigma));
+  k.A = sc.A;
+  k.alpha = sc.alpha;
+  k.beta = sc.beta;
+  if (cudaMemsetAsync(zero, 0, bytes, s) != cudaSuccess ||
+      launch_kx(mode, tile, k, (int)((ns + kKxWarps - 1) / kKxWarps), s) != cudaSuccess)
+    return GA_ERR_CUDA;
+  if (!stats) return GA_OK;
+  int32_t *hst = (int32_t *)pinned_scratch();
+  if (cudaEventRecord(ev.e1, s) != cudaSuccess ||
+      cudaMemcpyAsync(hst, k.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaStreamSynchronize(s) != cudaSuccess)
+    return GA_ERR_CUDA;
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, ev.e0, ev.e1);
+  std::memset(stats, 0, sizeof(*stats));
+  stats->cells = m * n;
+  stats->pairs = stats->pairs_int16 = 1;
+  stats->kernel_ms = stats->dp_ms = ms;
+  stats->dp_launches = stats->launches = 1;
+  stats->status = hst[0];
+  return GA_OK;
 }
 
 int batch_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
@@ -1244,8 +1387,10 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
       return GA_ERR_CUDA;
     for (int32_t i = 0; i < n_now; ++i) {
       const int64_t *f = &hinfo[(size_t)i * 4];
-      rc = sv_align_pair(q_codes + f[0], f[1], t_codes + f[2], f[3], c.sc.A, c.sc.mat, c.sc.alpha, c.sc.beta,
-                         GA_LOCAL, scores + ids[i], c.s, nullptr);
+      rc = std::max(c.sc.smax, 0) + c.sc.alpha <= kKxMaxStep
+               ? kx_align_pair(q_codes + f[0], f[1], t_codes + f[2], f[3], c.sc, GA_LOCAL, scores + ids[i], c.s, nullptr)
+               : sv_align_pair(q_codes + f[0], f[1], t_codes + f[2], f[3], c.sc.A, c.sc.mat, c.sc.alpha, c.sc.beta,
+                               GA_LOCAL, scores + ids[i], c.s, nullptr);
       if (rc) return rc;
     }
     c.pairs32 += n_now;
@@ -1449,6 +1594,7 @@ int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, cons
   pp.status = &P.small->status;
   pp.cells = &P.small->cells;
   pp.rmax_long = &P.small->rmax_long;
+  pp.long_sums = &P.small->long_sums;
   plan_kernel<<<vb, 256, 0, s>>>(pp);
   hist_kernel<<<vb, 256, 0, s>>>(P.keys, npairs, P.hist);
   scan_partials_kernel<<<kScanTiles, kScanTile, 0, s>>>(P.hist, P.small->scan_partials);
@@ -1975,8 +2121,11 @@ int ga_align_long(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, cons
     if (m >= (1ll << 30) || n >= (1ll << 30) ||
         2 * (int64_t)sc.alpha + (int64_t)sc.beta * (m + n) + 127 * mn >= (1ll << 30))
       return GA_ERR_RANGE;
-    // every strip of 512 columns on its own warp, a few rows behind its
-    // left neighbour (up to 65536 residues); longer: one warp per pair
+    // every strip of columns on its own warp, about a hundred rows behind its
+    // left neighbour (relative int16 cells); other scorings in int32 strips of
+    // 512 columns up to 65536 residues, longer on one warp
+    if (m > 0 && n > 0 && std::max(m, n) <= 65536 && std::max(sc.smax, 0) + sc.alpha <= kKxMaxStep)
+      return kx_align_pair(q, m, t, n, sc, mode, score, s, stats);
     if (m <= 65536 && n <= 65536)
       return sv_align_pair(q, m, t, n, sc.A, sc.mat, sc.alpha, sc.beta, mode, score, s, stats);
   }

@@ -72,6 +72,13 @@ struct CellS32 {
   static __device__ __forceinline__ T splat(int v) { return v; }
 };
 
+// Nanoseconds of the GPU's global timer (limits of the device-side waits).
+__device__ __forceinline__ uint64_t sv_now() {
+  uint64_t v;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(v));
+  return v;
+}
+
 // Device status word helpers: first error wins.
 __device__ __forceinline__ void set_status(int32_t *status, int code) {
   if (status) atomicCAS(status, 0, code);

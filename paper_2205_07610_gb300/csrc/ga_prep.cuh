@@ -14,6 +14,7 @@
 #pragma once
 
 #include "ga_common.cuh"
+#include "ga_kx.h"
 
 namespace ga {
 
@@ -28,6 +29,13 @@ struct BinTable {
   int w16[kBins];
   int n32;
   int w32[kBins];
+};
+
+// Sizes of the strip launch over the long-class pairs (ga_strip.cuh): sum of
+// (shorter sequence + 1), and the strips of every width.
+struct LongSums {
+  unsigned long long rows;
+  int32_t strips[kKxWidths], pad;
 };
 
 struct PlanParams {
@@ -50,6 +58,7 @@ struct PlanParams {
   int32_t *status;
   unsigned long long *cells;  // sum m*n over valid pairs
   int32_t *rmax_long;         // max rows over long-class pairs
+  LongSums *long_sums;        // sizes of the strip launch of the long class
 };
 
 // 2-bit codes of the 4 bytes of x (low 2 bits of each byte) in 8 bits.
@@ -212,7 +221,8 @@ __device__ __forceinline__ int global_gap(int alpha, int beta, int64_t len) {
 }
 
 // One pair (batch) or (query, target) combination (cross chunk).
-__device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigned long long &my_cells) {
+__device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigned long long &my_cells,
+                                         int &long_rows, int &long_cols) {
   const int64_t qi = p.nt ? p.q0 + i / p.nt : i;
   const int64_t ti = p.nt ? i % p.nt : i;
   const int64_t m = p.q_off[qi + 1] - p.q_off[qi];
@@ -264,7 +274,10 @@ __device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigne
         if (ok16) { cls = kClassInter16; bin = b16; }
         else if (b32 >= 0) { cls = kClassInter32; bin = b32; }
       }
-      if (cls == kClassLong) atomicMax(p.rmax_long, (int)R);
+      if (cls == kClassLong) {
+        long_rows = (int)C;
+        long_cols = (int)R;
+      }
       inf = make_int4((int)R, (int)C, swap, (int)cls);
       const int64_t rb = R < 1536 ? R : (1536 + ((R - 1536) >> 6) < kRBuckets - 1 ? 1536 + ((R - 1536) >> 6) : kRBuckets - 1);
       key = (uint32_t)(((cls * kBins + bin) * kRBuckets) + (kRBuckets - 1 - rb));
@@ -277,7 +290,25 @@ __device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigne
 __global__ void plan_kernel(PlanParams p) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long my_cells = 0;
-  if (i < p.npairs) plan_one(p, i, my_cells);
+  int long_rows = 0, long_cols = 0;
+  if (i < p.npairs) plan_one(p, i, my_cells, long_rows, long_cols);
+  if (__any_sync(0xffffffffu, long_cols != 0)) {
+    const unsigned cmax = __reduce_max_sync(0xffffffffu, (unsigned)long_cols);
+    // 32 x (2^30 + 1) needs more than 32 bits
+    unsigned long long rows = long_cols ? (unsigned long long)long_rows + 1 : 0;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, off);
+    unsigned strips[kKxWidths];
+#pragma unroll
+    for (int w = 0; w < kKxWidths; ++w)
+      strips[w] = __reduce_add_sync(0xffffffffu, ((unsigned)long_cols + kx_width(w) - 1) / kx_width(w));
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(p.rmax_long, (int)cmax);
+      atomicAdd(&p.long_sums->rows, rows);
+#pragma unroll
+      for (int w = 0; w < kKxWidths; ++w) atomicAdd(&p.long_sums->strips[w], (int)strips[w]);
+    }
+  }
   // one atomic per warp for the cell count
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) my_cells += __shfl_xor_sync(0xffffffffu, my_cells, off);

@@ -118,11 +118,6 @@ struct SvParams {
                        // launches of one pair, whose strips each have a scheduler to themselves
 };
 
-__device__ __forceinline__ uint64_t sv_now() {
-  uint64_t v;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(v));
-  return v;
-}
 __device__ __forceinline__ int sv_ld_acquire(const int32_t *p) {
   int v;
   asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
