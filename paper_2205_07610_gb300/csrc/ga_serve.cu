@@ -33,14 +33,13 @@ cudaError_t sv_prepare_launch(size_t smem, int *blocks_per_sm) {
 __global__ void sv_oneshot_init_kernel(SvRequest *rq, SvScoring *sc_out, const SvScoring sc,
                                        const uint8_t *q, const uint8_t *t, int2 *edges, int32_t *out,
                                        int m, int n, int mode, int nstrips, int2 *tasks,
-                                       unsigned long long *ctr, unsigned long long *cont_seq,
-                                       int32_t *stop) {
+                                       SvCtl *ctl, unsigned long long *cont_seq, int32_t *stop) {
   const int i = threadIdx.x;
   for (int k = i; k < kSvMaxStrips; k += blockDim.x) {
     rq->progress[k] = 0;
     cont_seq[k] = 0;
   }
-  if (i < 8) ctr[i] = 0;
+  for (int k = i; k < (int)(sizeof(SvCtl) / sizeof(int32_t)); k += blockDim.x) reinterpret_cast<int32_t *>(ctl)[k] = 0;
   if (i == 0) {
     tasks[0] = make_int2(0, 0);  // strip 0; the strips after it come as continuations
     *sc_out = sc;
@@ -61,19 +60,32 @@ __global__ void sv_oneshot_init_kernel(SvRequest *rq, SvScoring *sc_out, const S
   }
   __syncthreads();
   if (i == 0) {
-    ctr[1] = 1;  // tail: one task
-    ctr[3] = 1;  // one request admitted
+    ctl->tail.v = 1;      // one task
+    ctl->admitted.v = 1;  // of one request
   }
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Packed strips keep relative int16 cells exact while sigma_max + alpha <=
-// kSvPkMaxStep.
-int sv_packed_ok(int A, const int8_t *matrix, int alpha) {
+// Fills in what the packed strips read: whether the scoring is exact in relative
+// int16 cells, table words and score vectors of both orientations.
+void sv_set_scoring(SvScoring &sc, int A, const int8_t *matrix, int alpha, int beta) {
+  sc.A = A;
+  sc.alpha = alpha;
+  sc.beta = beta;
+  std::memcpy(sc.sigma, matrix, (size_t)(A * A));
   int smax = 0;
   for (int i = 0; i < A * A; ++i) smax = std::max(smax, (int)matrix[i]);
-  return smax + alpha <= kSvPkMaxStep ? 1 : 0;
+  sc.packed = smax + alpha <= kKxMaxStep ? 1 : 0;
+  for (int x = 0; x < A; ++x)
+    for (int c = 0; c < A; ++c) {
+      sc.vec[0][x][c] = matrix[c * A + x];  // column x is a target residue
+      sc.vec[1][x][c] = matrix[x * A + c];
+      if (A <= 4) {
+        sc.tables[0][x] |= (uint32_t)(uint8_t)matrix[x * A + c] << (8 * c);
+        sc.tables[1][x] |= (uint32_t)(uint8_t)matrix[c * A + x] << (8 * c);
+      }
+    }
 }
 
 }  // namespace
@@ -88,15 +100,11 @@ int sv_align_pair(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, int 
                   int alpha, int beta, int mode, int32_t *score, cudaStream_t s, ga_stats *stats) {
   if (m > kSvMaxLen || n > kSvMaxLen || A < 1 || A > 31) return GA_ERR_ARG;
   SvScoring sc{};
-  sc.A = A;
-  sc.alpha = alpha;
-  sc.beta = beta;
-  std::memcpy(sc.sigma, matrix, (size_t)(A * A));
-  sc.packed = sv_packed_ok(A, matrix, alpha);
+  sv_set_scoring(sc, A, matrix, alpha, beta);
   const int nstrips = sv_strips_for(m, n);
   const int64_t R = m < n ? m : n;
   const size_t o_sc = 0, o_rq = align256(o_sc + sizeof(SvScoring));
-  const size_t o_ht = align256(o_rq + sizeof(SvRequest)), o_stop = o_ht + 8 * sizeof(unsigned long long);
+  const size_t o_ht = align256(o_rq + sizeof(SvRequest)), o_stop = o_ht + sizeof(SvCtl);
   const size_t o_cseq = align256(o_stop + sizeof(int32_t));
   const size_t o_cont = align256(o_cseq + sizeof(unsigned long long) * kSvMaxStrips);
   const size_t o_tasks = align256(o_cont + sizeof(int2) * kSvMaxStrips);
@@ -106,7 +114,7 @@ int sv_align_pair(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, int 
   if (pool_malloc((void **)&base, bytes, s) != cudaSuccess) return GA_ERR_OOM;
   SvScoring *dsc = (SvScoring *)(base + o_sc);
   SvRequest *rq = (SvRequest *)(base + o_rq);
-  unsigned long long *ht = (unsigned long long *)(base + o_ht);
+  SvCtl *ctl = (SvCtl *)(base + o_ht);
   int32_t *stop = (int32_t *)(base + o_stop);
   int2 *tasks = (int2 *)(base + o_tasks);
   int2 *edges = (int2 *)(base + o_edges);
@@ -127,29 +135,22 @@ int sv_align_pair(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, int 
     cudaEventRecord(e0, s);
   }
   sv_oneshot_init_kernel<<<1, 128, 0, s>>>(rq, dsc, sc, q, t, edges, score, (int)m, (int)n, mode, nstrips,
-                                           tasks, ht, cseq, stop);
+                                           tasks, ctl, cseq, stop);
   SvParams p{};
   p.req = rq;
   p.scorings = dsc;
   p.tasks = tasks;
   p.task_cap = 1;
-  p.head = ht;
-  p.tail = ht + 1;
+  p.ctl = ctl;
   p.comp = nullptr;
   p.comp_cap = 1;
-  p.comp_count = nullptr;
   p.stop = stop;
   p.cont = cont;
   p.cont_seq = cseq;
   p.cont_cap = kSvMaxStrips;
-  p.cont_head = ht + 5;
-  p.cont_tail = ht + 6;
-  p.admitted = ht + 3;
-  p.completed = ht + 4;
   p.idle_ns = 0;
   p.wait_ns = 10ll * 1000 * 1000 * 1000;
   p.prof_bytes = (sc.A + 1) * kSvW;
-  p.short_chain = 1;  // one pair: each strip warp has a scheduler to itself
   const int grid = std::max(1, std::min((nstrips + kSvWarps - 1) / kSvWarps, nsm * std::max(occ, 1)));
   ks_kernel<<<grid, 32 * kSvWarps, smem, s>>>(p);
   int rc = cudaGetLastError() == cudaSuccess ? GA_OK : GA_ERR_CUDA;
@@ -234,7 +235,7 @@ struct ga_server {
   ga::SvRequest *req = nullptr;
   ga::SvScoring *scorings = nullptr;
   int2 *tasks = nullptr;
-  unsigned long long *ctr = nullptr;  // head, tail, comp_count, admitted, completed, cont head, cont tail
+  ga::SvCtl *ctl = nullptr;
   int2 *cont = nullptr;               // continuation ring (req_cap entries)
   unsigned long long *cont_seq = nullptr;
   // host (pinned, mapped where the kernel reads or writes it)
@@ -404,9 +405,9 @@ bool sched_tick(ga_server *S) {
     const unsigned long long new_tail = S->tail + (unsigned long long)ntasks;
     S->stage_tail[0] = new_tail;
     S->stage_tail[1] = (unsigned long long)(S->req_seq + (int64_t)admit.size());  // admitted
-    cudaMemcpyAsync(S->ctr + 1, S->stage_tail, sizeof(unsigned long long), cudaMemcpyHostToDevice,
+    cudaMemcpyAsync(&S->ctl->tail.v, S->stage_tail, sizeof(unsigned long long), cudaMemcpyHostToDevice,
                     S->feed);
-    cudaMemcpyAsync(S->ctr + 3, S->stage_tail + 1, sizeof(unsigned long long), cudaMemcpyHostToDevice,
+    cudaMemcpyAsync(&S->ctl->admitted.v, S->stage_tail + 1, sizeof(unsigned long long), cudaMemcpyHostToDevice,
                     S->feed);
     const bool ok = cudaStreamSynchronize(S->feed) == cudaSuccess;
     const int64_t t_admit = S->now_ns();
@@ -437,15 +438,13 @@ bool sched_tick(ga_server *S) {
     p.scorings = S->scorings;
     p.tasks = S->tasks;
     p.task_cap = S->task_cap;
-    p.head = S->ctr;
-    p.tail = S->ctr + 1;
+    p.ctl = S->ctl;
     SvCompletion *comp_d = nullptr;
     int32_t *stop_d = nullptr;
     cudaHostGetDevicePointer((void **)&comp_d, S->comp_h, 0);
     cudaHostGetDevicePointer((void **)&stop_d, S->stop_h, 0);
     p.comp = comp_d;
     p.comp_cap = S->req_cap;
-    p.comp_count = S->ctr + 2;
     p.stop = stop_d;
     p.idle_ns = S->idle_ns;
     p.wait_ns = 10ll * 1000 * 1000 * 1000;
@@ -453,10 +452,6 @@ bool sched_tick(ga_server *S) {
     p.cont = S->cont;
     p.cont_seq = S->cont_seq;
     p.cont_cap = S->req_cap;
-    p.cont_head = S->ctr + 5;
-    p.cont_tail = S->ctr + 6;
-    p.admitted = S->ctr + 3;
-    p.completed = S->ctr + 4;
     ks_kernel<<<S->grid, 32 * kSvWarps, S->smem, S->kstream>>>(p);
     if (cudaGetLastError() != cudaSuccess) S->sched_error = GA_ERR_CUDA;
     S->kernel_running = true;
@@ -583,7 +578,7 @@ int ga_server_create(const ga_server_config *cfg, ga_server **out) {
             cudaMalloc((void **)&S->req, sizeof(SvRequest) * (size_t)S->req_cap) == cudaSuccess &&
             cudaMalloc((void **)&S->scorings, sizeof(SvScoring) * GA_SERVE_MAX_SCORINGS) == cudaSuccess &&
             cudaMalloc((void **)&S->tasks, sizeof(int2) * (size_t)S->task_cap) == cudaSuccess &&
-            cudaMalloc((void **)&S->ctr, 8 * sizeof(unsigned long long)) == cudaSuccess &&
+            cudaMalloc((void **)&S->ctl, sizeof(SvCtl)) == cudaSuccess &&
             cudaMalloc((void **)&S->cont, sizeof(int2) * (size_t)S->req_cap) == cudaSuccess &&
             cudaMalloc((void **)&S->cont_seq, sizeof(unsigned long long) * (size_t)S->req_cap) == cudaSuccess &&
             cudaHostAlloc((void **)&S->comp_h, sizeof(SvCompletion) * (size_t)S->req_cap,
@@ -602,7 +597,7 @@ int ga_server_create(const ga_server_config *cfg, ga_server **out) {
   }
   std::memset(S->comp_h, 0, sizeof(SvCompletion) * (size_t)S->req_cap);
   *S->stop_h = 0;
-  if (cudaMemset(S->ctr, 0, 8 * sizeof(unsigned long long)) != cudaSuccess ||
+  if (cudaMemset(S->ctl, 0, sizeof(SvCtl)) != cudaSuccess ||
       cudaMemset(S->cont_seq, 0, sizeof(unsigned long long) * (size_t)S->req_cap) != cudaSuccess) {
     ga_server_destroy(S.release());
     return GA_ERR_CUDA;
@@ -630,14 +625,9 @@ int ga_server_add_scoring(ga_server *S, const ga_scoring *sc, int32_t *scoring_i
   if (sc->gap_open <= 0 || sc->gap_extend <= 0 || sc->gap_extend > sc->gap_open || sc->gap_open > 4096)
     return GA_ERR_ARG;
   SvScoring h{};
-  h.A = sc->alphabet_size;
-  h.alpha = sc->gap_open;
-  h.beta = sc->gap_extend;
-  for (int i = 0; i < h.A * h.A; ++i) {
+  for (int i = 0; i < sc->alphabet_size * sc->alphabet_size; ++i)
     if (sc->matrix[i] < -127) return GA_ERR_ALPHABET;
-    h.sigma[i] = sc->matrix[i];
-  }
-  h.packed = sv_packed_ok(h.A, h.sigma, h.alpha);
+  sv_set_scoring(h, sc->alphabet_size, sc->matrix, sc->gap_open, sc->gap_extend);
   std::lock_guard<std::mutex> lk(S->mu);
   if ((int)S->sc_host.size() >= GA_SERVE_MAX_SCORINGS) return GA_ERR_ARG;
   if (S->st.submitted > 0 && h.A > S->max_A) return GA_ERR_ARG;  // profile size is fixed once serving
@@ -751,7 +741,7 @@ int ga_server_destroy(ga_server *S) {
   cudaFree(S->req);
   cudaFree(S->scorings);
   cudaFree(S->tasks);
-  cudaFree(S->ctr);
+  cudaFree(S->ctl);
   cudaFree(S->cont);
   cudaFree(S->cont_seq);
   cudaFreeHost(S->comp_h);

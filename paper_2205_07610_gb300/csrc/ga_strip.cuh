@@ -111,8 +111,13 @@ struct StripState {
   uint32_t best;  // local: running maximum, relative
 };
 
-// Row update.  FC: the one-op column chain of pk_row_fc (local and global mode),
-// with local mode's zero taken into X(j) = max(Hdiag + sigma, E, Z).
+// Row update.  FC: a one-op chain across the columns (local and global mode,
+// where every column's gap open alpha >= beta).  With X(j) = max(Hdiag + sigma, E
+// [, Z in local mode]) the H of a column is max(X(j), F(j)), and since F(j) -
+// alpha <= F(j) - beta the gap entering the next column is F(j+1) = max(F(j) -
+// beta, X(j) - alpha): it no longer waits for H(j).  One more ALU and one more FMA
+// operation per packed column, for a chain of one operation per column instead of
+// three.
 template <int MODE, int K, bool FC, class SigFn, class NaFn>
 __device__ __forceinline__ uint32_t strip_row(StripState<K> &s, uint32_t NB, uint32_t NAc, SigFn SIG, NaFn NA) {
   static_assert(!FC || MODE != kModeSemi, "semi-global frees the last column's gap open");
@@ -149,21 +154,33 @@ __device__ __forceinline__ uint32_t strip_row(StripState<K> &s, uint32_t NB, uin
 template <int K>
 constexpr int kx_prof_row = 64 * K;  // bytes of a profile row: low half, then high half
 
+// One pair as the strip function sees it: rows and columns, the scoring, the
+// edge words of rows 0 .. R.
 struct KXView {
   const uint8_t *row, *col;
   int R, C, sw, nstrips;
+  int A, alpha, beta;
   unsigned long long *edges;
 };
 
-template <int MODE, int K, bool FC, bool PROF>
-__device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int s, int t, uint2 *ring,
-                                        uint32_t *in, uint2 *out, uint8_t *prof, const uint32_t *sig,
-                                        int &status) {
+struct KXNoHook {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+
+// Strip s of a pair; returns its contribution to the score (local: best H; semi-
+// global: max of row R; global: H(R, C) in the last strip).  tables: the table
+// words of the 4 row codes (no profile); sig: the score vectors of the column
+// residues, SIGW words apart (profile).  on_rows(n) is called when rows 1 .. n of
+// the right edge have been written.
+template <int MODE, int K, bool FC, bool PROF, int SIGW, class OnRows>
+__device__ __forceinline__ int kx_strip(const KXView &v, int s, int t, uint2 *ring, uint32_t *in, uint2 *out,
+                                        uint8_t *prof, const uint32_t *sig, const uint32_t *tables, int &status,
+                                        OnRows on_rows) {
   constexpr int WH = 32 * K, W = 64 * K, NQ = K / 4;
   constexpr unsigned FULL = 0xffffffffu;
   static_assert(K % 4 == 0, "profile words");
   static_assert(kKxMaxStep * (kKwRenorm + 2 * K + 8) < 32000 - 256, "relative int16 cells of this tile width");
-  const int R = v.R, C = v.C, A = p.A, alpha = p.alpha, beta = p.beta;
+  const int R = v.R, C = v.C, A = v.A, alpha = v.alpha, beta = v.beta;
   const int col0 = s * W, ncol = ::min(W, C - col0);
   const bool edge_out = s + 1 < v.nstrips;
   const uint32_t NB = pk16(-beta, -beta), NAc = pk16(-alpha, -alpha);
@@ -171,6 +188,8 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
   auto h0 = [&](int c) -> int { return (MODE == kModeGlobal && c > 0) ? -alpha - beta * (c - 1) : 0; };
   int bad = 0;  // a residue code >= A
 
+  // (codes are read past L1: the server's buffers are refilled while its kernel
+  // runs)
   // ---- columns: selectors, or the strip's profile ---------------------------
   uint32_t sel[PROF ? 1 : K];
   uint32_t na[MODE == kModeSemi ? K : 1];
@@ -180,7 +199,7 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
   for (int j = 0; j < K; ++j) {
     const int c0 = t * K + j, c1 = c0 + WH;
     if constexpr (!PROF) {
-      const int x0 = c0 < ncol ? (int)__ldg(v.col + col0 + c0) : -1, x1 = c1 < ncol ? (int)__ldg(v.col + col0 + c1) : -1;
+      const int x0 = c0 < ncol ? (int)__ldcg(v.col + col0 + c0) : -1, x1 = c1 < ncol ? (int)__ldcg(v.col + col0 + c1) : -1;
       bad |= (x0 >= A) | (x1 >= A);
       // pad columns replicate a table byte's sign: sigma in {0, -1}
       const uint32_t n0 = x0 >= 0 ? (uint32_t)(x0 & 3) : 8u, n0s = x0 >= 0 ? (uint32_t)((x0 & 3) + 8) : 8u;
@@ -205,9 +224,9 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
       const uint32_t *sg[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int x = cb + i < ncol ? (int)__ldg(v.col + col0 + cb + i) : A;
+        const int x = cb + i < ncol ? (int)__ldcg(v.col + col0 + cb + i) : A;
         bad |= cb + i < ncol && x >= A;
-        sg[i] = sig + ::min(x, A) * kKxSigRow;
+        sg[i] = sig + ::min(x, A) * SIGW;
       }
       uint32_t *dst = pw + (q / NQ) * (WH / 4) + (q % NQ) * 32 + t;
 #pragma unroll 1
@@ -233,7 +252,7 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
                              : (MODE == kModeGlobal) ? 0x01010101u * (uint32_t)(uint8_t)(-beta) : 0u;
   auto read_code = [&](int bb) -> int {  // row 32bb + 1 + t, -1 past the last
     const int r = 32 * bb + t;
-    return r < R ? (int)__ldg(v.row + r) : -1;
+    return r < R ? (int)__ldcg(v.row + r) : -1;
   };
   auto row_word = [&](int c) -> uint32_t {
     if constexpr (PROF) {
@@ -241,7 +260,7 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
       return (uint32_t)((c < 0 || c >= A) ? A : c) * (uint32_t)W;
     } else {
       bad |= c >= A;
-      return c < 0 ? 0u : p.tables[(v.sw ? 8 : 0) + (c & 3)];
+      return c < 0 ? 0u : tables[c & 3];
     }
   };
   auto put_row = [&](int x, uint32_t lo, uint32_t hi) {
@@ -321,7 +340,10 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
 
   for (int it0 = 0; it0 < nit; it0 += 32) {
     __syncwarp();
-    if (edge_out) flush(it0);
+    if (edge_out) {
+      flush(it0);
+      on_rows(it0 - 63);
+    }
     if ((it0 & (kKwRenorm - 1)) == 0 && it0 > 0) {
       // move each half's base to its current H of the first column
       const int d0 = lo16(st.H[0]), d1 = hi16(st.H[0]);
@@ -442,6 +464,7 @@ __device__ __forceinline__ int kx_strip(const KXParams &p, const KXView &v, int 
   if (edge_out) {  // rows of the last two batches (nit = R + 63: rows up to R)
     const int last0 = ((nit + 31) / 32) * 32;
     flush(last0);
+    on_rows(R);
   }
   if (__any_sync(FULL, bad)) status = GA_ERR_RESIDUE;
   if (gave_up) status = GA_ERR_TIMEOUT;
@@ -507,9 +530,13 @@ __global__ void __launch_bounds__(32 * kKxWarps, 1) kx_kernel(const __grid_const
     v.col = v.sw ? p.q_codes + qs : p.t_codes + ts;
     v.nstrips = (v.C + 64 * K - 1) / (64 * K);
     v.edges = p.edges + eo;
+    v.A = p.A;
+    v.alpha = p.alpha;
+    v.beta = p.beta;
     int status = GA_OK;
-    const int val = kx_strip<MODE, K, FC, PROF>(p, v, s, t, ring_s[warp], in_s[warp], out_s[warp], prof,
-                                                   sig_s[PROF ? v.sw : 0], status);
+    const int val = kx_strip<MODE, K, FC, PROF, kKxSigRow>(v, s, t, ring_s[warp], in_s[warp], out_s[warp], prof,
+                                                           sig_s[PROF ? v.sw : 0], p.tables + (v.sw ? 8 : 0), status,
+                                                           KXNoHook{});
     if (t == 0) {
       KXPairState *ps = p.state + li;
       bool finish = v.nstrips == 1;
