@@ -24,8 +24,12 @@ namespace ga {
 
 namespace {
 
+// The kernel's shared-memory limit is one setting per device for every user of
+// the kernel (servers and single pairs): it is set to the largest profile, so that
+// no user lowers it below what another one launches with.
 cudaError_t sv_prepare_launch(size_t smem, int *blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(ks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(ks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)((size_t)kSvWarps * 32 * kSvW));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, ks_kernel, 32 * kSvWarps, smem);
 }
