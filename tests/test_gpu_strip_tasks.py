@@ -95,3 +95,31 @@ def test_single_pairs_and_scorings(mode):
             a, b = _related(rng, m, n, sc[0].shape[0])
             got = ga.align_long(torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda(), *sc, mode)
             assert int(got.item()) == oracle.score(a, b, *sc, mode), (k, m, n)
+
+
+@pytest.mark.parametrize("mode", MODES)
+def test_bases_that_move_far_at_the_last_rows(mode):
+    """Steep scorings (sigma_max + alpha = 128) on identical sequences: a base
+    moves by thousands per 128 rows, also while lane 0 is past the last row (its
+    left input is -inf there).  Batches and the server run strip tasks, plans the
+    one-warp kernel."""
+    rng = np.random.default_rng(11)
+    mat, alpha, beta = synth.dna_matrix(100, -100), 28, 1
+    seqs = [rng.integers(0, 4, n).astype(np.uint8) for n in range(960, 1100, 5)]
+    # a row sequence that ends where its alignment has just entered a strip
+    longer = [np.concatenate([s, rng.integers(0, 4, 150).astype(np.uint8)]) for s in seqs]
+    _check([(s, s.copy()) for s in seqs] + list(zip(seqs, longer)), (mat, alpha, beta), mode)
+    qc, qo = synth.pack_csr(seqs)
+    tc, to = synth.pack_csr(longer)
+    want, _ = oracle.batch(qc, qo, tc, to, mat, alpha, beta, mode, nthreads=NTHREADS)
+    with ga.Server(arena_bytes=1 << 26, idle_us=200) as srv:
+        sid = srv.add_scoring(mat, alpha, beta)
+        srv.submit(qc, qo, tc, to, MODES.index(mode), sid)
+        srv.drain(30_000)
+        got = np.sort(srv.poll(), order="id")
+    assert (got["score"] == want).all() and (got["status"] == 0).all()
+    qc, qo = synth.pack_csr(seqs)
+    d = [torch.from_numpy(a).cuda() for a in (qc, qo, qc.copy(), qo.copy())]
+    with ga.Plan(mat, alpha, beta, mode, len(seqs), len(qc), 1100) as plan:
+        got = plan.run(*d).cpu().numpy()
+    assert (got == [100 * len(s) for s in seqs]).all()
