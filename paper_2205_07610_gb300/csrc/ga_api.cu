@@ -18,6 +18,8 @@
 #include "ga_kx.h"
 #include "ga_launch.h"
 #include "ga_prep.cuh"
+#include "ga_reads.cuh"
+#include "ga_reads.h"
 #include "ga_strip_tasks.cuh"
 
 namespace ga {
@@ -176,7 +178,7 @@ struct Alloc {
 // Small pinned staging area for scalar readbacks (one per host thread).
 struct Pinned {
   void *p = nullptr;
-  Pinned() { cudaMallocHost(&p, 4096); }
+  Pinned() { cudaMallocHost(&p, 8192); }
   ~Pinned() {
     if (p) cudaFreeHost(p);
   }
@@ -192,6 +194,8 @@ struct Small {
   int32_t rmax_long;
   LongSums long_sums;
   unsigned long long cells;
+  int64_t ends[4];   // small batches: q_off[0], q_off[npairs], t_off[0], t_off[npairs]
+  int32_t left, pad1;  // small batches: pairs too long for the one-launch kernel
   int32_t rerun_total;
   int32_t pad0;
   int32_t ranges[2 * kClassesSorted * kBins];
@@ -209,6 +213,8 @@ struct Readback {
   int32_t rmax_long;
   LongSums long_sums;
   unsigned long long cells;
+  int64_t ends[4];   // small batches: q_off[0], q_off[npairs], t_off[0], t_off[npairs]
+  int32_t left, pad1;  // small batches: pairs too long for the one-launch kernel
   int32_t rerun_total;
   int32_t pad0;
   int32_t ranges[2 * kClassesSorted * kBins];
@@ -295,11 +301,16 @@ int setup(Call &c) {
     return GA_ERR_CUDA;
   c.dna = c.sc.A <= 4;
   c.small = c.al.get<Small>(1);
-  c.hist = c.al.get<int32_t>(kNumKeys);
-  c.cursor = c.al.get<int32_t>(kNumKeys);
   if (c.al.failed) return GA_ERR_OOM;
   if (cudaMemsetAsync(c.small, 0, sizeof(Small), c.s) != cudaSuccess) return GA_ERR_CUDA;
   return GA_OK;
+}
+
+// The counting sort's buffers.
+int setup_sort(Call &c) {
+  c.hist = c.al.get<int32_t>(kNumKeys);
+  c.cursor = c.al.get<int32_t>(kNumKeys);
+  return c.al.failed ? GA_ERR_OOM : GA_OK;
 }
 
 // Validate + pack one sequence set.  Reads back the total residue count.
@@ -426,6 +437,7 @@ struct ChunkPlan {
   int64_t npairs = 0, nt = 0, q0 = 0;
   int32_t *scores = nullptr;
   int force_long = 0;
+  int32_t done_len = 0;
   Small *sm = nullptr;
   int32_t *hist = nullptr, *cursor = nullptr;
   uint32_t *keys = nullptr;
@@ -467,6 +479,7 @@ int plan_enqueue(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   pp.sigma_max = c.sc.smax;
   pp.sigma_min = c.sc.smin;
   pp.dna = c.dna && !p.force_long;
+  pp.done_len = p.done_len;
   pp.bins = make_bins();
   pp.scores = p.scores;
   pp.keys = p.keys;
@@ -489,7 +502,7 @@ int plan_enqueue(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
 // Bin populations and longest long-class pair of n plans: one copy each,
 // one synchronisation.
 int plan_readback(Call &c, ChunkPlan *ps, int n) {
-  static_assert(8 * sizeof(Readback) <= 4096, "pinned scratch holds the readbacks of 8 plans");
+  static_assert(8 * sizeof(Readback) <= 8192, "pinned scratch holds the readbacks of 8 plans");
   Readback *rb = (Readback *)pinned_scratch();
   bool any = false;
   for (int k = 0; k < n; ++k) {
@@ -860,6 +873,66 @@ struct Events {
   }
 };
 
+// Batches that go to the one-launch kernel first, and plans whose capacity it
+// takes.  Its strips pad a pair to 256, 512 or 768 columns, so it is the slower
+// kernel once the chip is full.  GB300, us a call, planned / one launch: 1,000
+// pairs of 150 residues 183 / 70, 4,000 of 100..300 349 / 164, 8,000 of 250..500
+// 480 / 444, 16,000 of 250..500 657 / 787.  A plan's default tuning runs its bins
+// in line, which loses to one launch for longer: 1,000 of 100..300 553 / 58,
+// 16,000 of 250..500 1,321 / 731, 32,000 of 150 370 / 339.
+constexpr int64_t kKrPairs = 8192;
+constexpr int64_t kKrPlanPairs = 32768;
+
+bool kr_scoring(const Scoring &sc) { return sc.A <= 4 && std::max(sc.smax, 0) + sc.alpha <= kKxMaxStep; }
+
+KRParams make_kr(const Scoring &sc, const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
+                 const int64_t *t_off, int64_t npairs, int32_t *scores, Small *small) {
+  KRParams k{};
+  k.q_codes = q_codes;
+  k.t_codes = t_codes;
+  k.q_off = q_off;
+  k.t_off = t_off;
+  k.npairs = (int32_t)npairs;
+  std::memcpy(k.tables, sc.tables, sizeof(k.tables));
+  k.A = sc.A;
+  k.alpha = sc.alpha;
+  k.beta = sc.beta;
+  k.scores = scores;
+  k.status = &small->status;
+  k.cells = &small->cells;
+  k.computed = &small->ranges[1];  // the population of the first packed bin
+  k.left = &small->left;
+  k.ends = small->ends;
+  return k;
+}
+
+// A small batch in one launch per mode.  *left: pairs too long for it, which
+// have to be planned; *qr, *tr then hold the residue ranges.
+int small_batch(Call &c, const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
+                const int64_t *t_off, int64_t npairs, const int32_t *modes, int nmodes, int32_t *scores,
+                int64_t score_stride, int32_t *left, KnownRange *qr, KnownRange *tr) {
+  for (int k = 0; k < nmodes; ++k) {
+    const KRParams kp = make_kr(c.sc, q_codes, q_off, t_codes, t_off, npairs, scores + (size_t)k * (size_t)score_stride,
+                                c.small);
+    c.dp_begin();
+    const cudaError_t e = launch_kr(modes[k], kp, c.s);
+    c.dp_end();
+    if (e != cudaSuccess) return GA_ERR_CUDA;
+  }
+  Readback *rb = (Readback *)pinned_scratch();
+  if (cudaMemcpyAsync(rb, c.small, sizeof(Readback), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
+      cudaStreamSynchronize(c.s) != cudaSuccess)
+    return GA_ERR_CUDA;
+  *left = rb->left;
+  c.pairs16 = rb->ranges[1];
+  qr->known = tr->known = true;
+  qr->start = rb->ends[0];
+  qr->total = rb->ends[1];
+  tr->start = rb->ends[2];
+  tr->total = rb->ends[3];
+  return GA_OK;
+}
+
 // Independent pairs in one or more modes: both sequence sets are validated
 // and packed once, then every mode is planned and aligned on the packed
 // copies; the scores of mode k go to scores + k * score_stride.
@@ -879,6 +952,15 @@ int batch_modes_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t
   c.timing = stats != nullptr;
   Events ev(stats != nullptr, c.s);
   if ((rc = setup(c))) return rc;
+  int32_t done_len = 0;
+  if (npairs > 0 && npairs <= kKrPairs && !force_long && kr_scoring(c.sc)) {
+    int32_t left = 0;
+    rc = small_batch(c, q_codes, q_off, t_codes, t_off, npairs, modes, nmodes, scores, score_stride, &left, &qr, &tr);
+    if (rc) return rc;
+    if (left == 0) return finish(c, stats, ev.e0, ev.e1, npairs * nmodes);
+    done_len = kKrMaxLen;
+  }
+  if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
   if ((rc = prepare_set(c, q_codes, q_off, npairs, &Q.packed, &Q.bad, &c.small->invalid_q, qr))) return rc;
   if ((rc = prepare_set(c, t_codes, t_off, npairs, &T.packed, &T.bad, &c.small->invalid_t, tr))) return rc;
@@ -891,6 +973,7 @@ int batch_modes_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t
     p.npairs = npairs;
     p.scores = scores + (size_t)k * (size_t)score_stride;
     p.force_long = force_long;
+    p.done_len = done_len;
     p.sm = k == 0 ? c.small : c.al.get<Small>(1);
     p.hist = k == 0 ? c.hist : c.al.get<int32_t>(kNumKeys);
     p.cursor = k == 0 ? c.cursor : c.al.get<int32_t>(kNumKeys);
@@ -1020,6 +1103,7 @@ struct BandRun {
 
   int prepare() {
     int rc;
+    if ((rc = setup_sort(c))) return rc;
     if ((rc = prepare_set(c, Q.codes, Q.off, npairs, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
     if ((rc = prepare_set(c, T.codes, T.off, npairs, &T.packed, &T.bad, &c.small->invalid_t))) return rc;
     keys = c.al.get<uint32_t>((size_t)npairs);
@@ -1235,6 +1319,7 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
                         const uint8_t *t_codes, const int64_t *t_off, int64_t nt, int32_t *scores,
                         ga_stats *stats, cudaEvent_t e0, cudaEvent_t e1) {
   int rc;
+  if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
   if ((rc = prepare_set(c, q_codes, q_off, nq, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
   uint32_t *t_packed5 = nullptr;
@@ -1262,7 +1347,7 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   std::vector<int64_t> hqo((size_t)nq + 1);
   std::vector<uint8_t> hqb((size_t)nq);
   Small *hs = (Small *)pinned_scratch();
-  static_assert(sizeof(Small) <= 4096, "pinned scratch holds the call's scalars");
+  static_assert(sizeof(Small) <= 8192, "pinned scratch holds the call's scalars");
   if (cudaMemcpyAsync(hqo.data(), q_off, sizeof(int64_t) * (size_t)(nq + 1), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
       cudaMemcpyAsync(hqb.data(), Q.bad, (size_t)nq, cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
       cudaMemcpyAsync(hs, c.small, sizeof(Small), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
@@ -1427,6 +1512,7 @@ struct PlanImpl {
   int occ16[kKaNumBins] = {}, occ32[kKaNumBins] = {}, occ16alt[kKaNumBins] = {};
   int occ_kb = 0, long_grid = 0;
   bool long_packed = false;
+  bool one_launch = false;  // capacity and scoring of the small-batch kernel (used while the tuning is the default)
   size_t long_smem = 0;
   Small *small = nullptr;
   int32_t *hist = nullptr, *cursor = nullptr;
@@ -1515,6 +1601,7 @@ int plan_create(const ga_scoring *scoring, int32_t mode, int64_t max_pairs, int6
                                       : mode == GA_GLOBAL ? blocks_per_sm_kb_global_prof(P->long_smem)
                                                           : blocks_per_sm_kb_semi_prof(P->long_smem));
   P->occ_kb = std::max(P->occ_kb, 1);
+  P->one_launch = kr_scoring(P->sc) && max_len <= kKrMaxLen && max_pairs <= kKrPlanPairs;
   P->long_grid = (int)std::min<int64_t>((int64_t)P->nsm * P->occ_kb, (max_pairs + kKbWarps - 1) / kKbWarps);
   P->bnd_stride = (int64_t)max_len + 128;
   P->small = P->alloc<Small>(1);
@@ -1545,6 +1632,11 @@ int plan_create(const ga_scoring *scoring, int32_t mode, int64_t max_pairs, int6
   return GA_OK;
 }
 
+bool default_tuning(const ga_tuning &t) {
+  const uint32_t all = (1u << kKaNumBins) - 1;
+  return t.tiles16 == all && t.tiles32 == all && t.concurrent == 0 && t.lanes_alt == 0;
+}
+
 // One run, enqueued on s with no host synchronisation and no allocation.
 int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
                  const int64_t *t_off, int64_t npairs, int32_t *scores, cudaStream_t s) {
@@ -1552,10 +1644,16 @@ int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, cons
   if (npairs > 0 && (!q_codes || !q_off || !t_codes || !t_off || !scores)) return GA_ERR_ARG;
   int cur = 0;
   if (cudaGetDevice(&cur) != cudaSuccess || cur != P.dev) return GA_ERR_ARG;
-  if (cudaMemsetAsync(P.small, 0, sizeof(Small), s) != cudaSuccess ||
-      cudaMemsetAsync(P.hist, 0, sizeof(int32_t) * kNumKeys, s) != cudaSuccess)
-    return GA_ERR_CUDA;
+  if (cudaMemsetAsync(P.small, 0, sizeof(Small), s) != cudaSuccess) return GA_ERR_CUDA;
   if (npairs == 0) return GA_OK;
+  if (P.one_launch && default_tuning(P.tune)) {
+    KRParams kp = make_kr(P.sc, q_codes, q_off, t_codes, t_off, npairs, scores, P.small);
+    kp.plan = 1;
+    kp.cap = P.max_res;
+    kp.max_len = P.max_len;
+    return launch_kr(P.mode, kp, s) == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+  }
+  if (cudaMemsetAsync(P.hist, 0, sizeof(int32_t) * kNumKeys, s) != cudaSuccess) return GA_ERR_CUDA;
   const int A = P.sc.A;
   const bool dna = A <= 4;
   const unsigned vb = (unsigned)((npairs + 255) / 256);
@@ -2088,6 +2186,7 @@ int ga_align_cross(const uint8_t *q_codes, const int64_t *q_off, int64_t nq, con
   if (nq == 0 || nt == 0) return finish(c, stats, ev.e0, ev.e1, 0);
   if (c.sc.A > 4 && mode == GA_LOCAL)
     return cross_protein_local(c, q_codes, q_off, nq, t_codes, t_off, nt, scores, stats, ev.e0, ev.e1);
+  if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
   if ((rc = prepare_set(c, q_codes, q_off, nq, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
   if ((rc = prepare_set(c, t_codes, t_off, nt, &T.packed, &T.bad, &c.small->invalid_t))) return rc;

@@ -51,6 +51,7 @@ struct PlanParams {
   int32_t alpha, beta;
   int32_t sigma_max, sigma_min;
   int32_t dna;                // alphabet packed 2-bit (<= 4 symbols)
+  int32_t done_len;           // pairs of at most this many residues each have their score (0: none)
   BinTable bins;
   int32_t *scores;
   uint32_t *keys;
@@ -239,6 +240,11 @@ __device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigne
     p.scores[i] = (p.mode == GA_GLOBAL) ? global_gap(p.alpha, p.beta, m + n) : 0;
   } else {
     const int64_t R = m >= n ? m : n, C = m >= n ? n : m;
+    if (R <= p.done_len) {
+      p.info[i] = inf;
+      p.keys[i] = key;
+      return;
+    }
     const int swap = m < n;
     const int64_t smax = p.sigma_max > 0 ? p.sigma_max : 0;
     const int64_t sabs = max(smax, (int64_t)(p.sigma_min < 0 ? -p.sigma_min : 0));
