@@ -233,8 +233,11 @@ int ga_align_long(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n,
  *            for pairs that ran as full DP (alphabets of more than 4
  *            symbols, where no banded kernel exists)
  *   w0     : entries < 0 are taken as 0
+ * The call decides an attempt by the pair's exact score where that is the
+ * faster way (S(w) = the exact score whenever that exceeds UB, and never
+ * above it); scores and w_used are those of the doubling in either case.
  * Errors as for ga_align_batch; stats->band_retries and ->banded_cells
- * count doublings and evaluated region cells.
+ * count the doublings and the region cells of the attempts.
  */
 int ga_align_banded(const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
                     const int64_t *t_off, int64_t npairs, const ga_scoring *scoring,

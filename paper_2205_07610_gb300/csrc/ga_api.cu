@@ -1,6 +1,7 @@
 // ga_api.cu -- the C ABI (include/gotoh_align.h): argument checks, workspace,
 // planning (encode, classify, length sort) and kernel dispatch.
 #include <algorithm>
+#include <cmath>
 #include <memory>
 #include <cstddef>
 #include <cstdio>
@@ -11,6 +12,7 @@
 #include "../../include/gotoh_band.h"
 #include "../../include/gotoh_plan.h"
 #include "ga_band.cuh"
+#include "ga_bandfull.cuh"
 #include "ga_banded.cuh"
 #include "ga_pool.h"
 #include "ga_prot.cuh"
@@ -204,6 +206,8 @@ struct Small {
   int32_t scan_partials[kScanTiles];
   int32_t invalid_q, invalid_t;
   unsigned long long band_retries, band_cells;
+  unsigned long long band_est;
+  int32_t hand_range[2], tie_range[2];  // band pairs decided by their exact score; attempts to run all the same
   int32_t max_rows;
   int32_t max_band_span;  // max over band pairs of max(m + 1, 128) x super-stages + m, saturated
 };
@@ -1086,6 +1090,10 @@ __global__ void bisect_final_kernel(int64_t npairs, const int32_t *lo, int32_t *
   if (i < npairs) w_min[i] = lo[i];
 }
 
+// Rows of a block's window beyond which a pair that failed is decided by its exact
+// score instead of the next attempt.
+constexpr int kBandHandLen = 1200;
+
 // A planned banded run (global mode, alphabets of <= 4 symbols): both sets
 // packed, pairs ordered by estimated band work, boundary buffers sized.
 struct BandRun {
@@ -1098,6 +1106,9 @@ struct BandRun {
   bool packed = false;  // packed int16x2 kernel (sigma_max + alpha <= kKzMaxStep)
   int64_t stride = 0;
   int2 *bnd = nullptr;
+  LongSums sums{};            // over the pairs to run: sizes of a strip launch,
+  int64_t longest = 0;        // the longest sequence,
+  double full_cells = 0, first_cells = 0;  // cells of the full matrices and (about) of the first attempts
   BandRun(Call &cc, const uint8_t *qc, const int64_t *qo, const uint8_t *tc, const int64_t *to, int64_t np)
       : c(cc), Q{qc, qo, nullptr, nullptr}, T{tc, to, nullptr, nullptr}, npairs(np) {}
 
@@ -1129,7 +1140,10 @@ struct BandRun {
     bp.keys = keys;
     bp.status = &c.small->status;
     bp.cells = &c.small->cells;
+    bp.sums = &c.small->long_sums;
+    bp.est = &c.small->band_est;
     bp.max_rows = &c.small->max_rows;
+    bp.max_len = &c.small->rmax_long;
     bp.max_span = &c.small->max_band_span;
     bp.stage_cols = kBandStageCols;
     const unsigned nb = (unsigned)((npairs + 255) / 256);
@@ -1141,16 +1155,20 @@ struct BandRun {
     scatter_kernel<<<nb, 256, 0, c.s>>>(keys, npairs, c.cursor, sorted);
     c.launches += 5;
     if (cudaGetLastError() != cudaSuccess) return GA_ERR_CUDA;
-    int32_t *h = (int32_t *)pinned_scratch();
-    if (cudaMemcpyAsync(h, &c.small->max_rows, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
+    const Small *h = (const Small *)pinned_scratch();
+    if (cudaMemcpyAsync((void *)h, c.small, sizeof(Small), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
         cudaStreamSynchronize(c.s) != cudaSuccess)
       return GA_ERR_CUDA;
-    max_rows = h[0];
+    max_rows = h->max_rows;
+    sums = h->long_sums;
+    longest = h->rmax_long;
+    full_cells = (double)h->cells;
+    first_cells = (double)h->band_est;
     if (max_rows > 0) {
       // the packed kernel numbers its iterations in int32: a pair runs at
       // most max(m + 1, 128) x super-stages + m + 64 of them; calls with
       // larger pairs take the int32 kernel, which runs one stage at a time
-      packed = std::max(c.sc.smax, 0) + c.sc.alpha <= kKzMaxStep && h[1] < kKzMaxSpan;
+      packed = std::max(c.sc.smax, 0) + c.sc.alpha <= kKzMaxStep && h->max_band_span < kKzMaxSpan;
       const int occ = std::max(packed ? blocks_per_sm_kz() : blocks_per_sm_kc(), 1);
       const int64_t want = (npairs + kKcWarps - 1) / kKcWarps;
       grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)c.nsm * occ));
@@ -1193,9 +1211,163 @@ struct BandRun {
     kc.bnd_stride = stride;
     kc.bis_lo = bis_lo;
     kc.bis_hi = bis_hi;
+    Full f;
+    if (packed && !bis_lo)
+      if (int rc = full_setup(f)) return rc;
+    if (f.on && full_first(default_w0, w0 != nullptr)) return full_run(f, kc, sorted, kc.range, nullptr);
+    f.on = f.on && few_pairs();
+    if (f.on) {
+      kc.hand_count = &c.small->hand_range[1];
+      kc.hand_list = f.list;
+      kc.hand_w = f.w_next;
+      kc.hand_len = kBandHandLen;
+    }
     c.dp_begin();
     const cudaError_t e = packed ? launch_kz(kc, grid, c.s) : launch_kc(kc, grid, c.s);
     c.dp_end();
+    if (e != cudaSuccess) return GA_ERR_CUDA;
+    return f.on ? full_run(f, kc, f.list, c.small->hand_range, f.w_next) : GA_OK;
+  }
+
+  // ---- pairs decided by their exact score (ga_bandfull.cuh) --------------------
+  struct Full {
+    bool on = false;
+    int tile = 0;
+    int64_t cap = 0;  // strip tasks of all pairs
+    size_t bytes = 0;
+    char *zero = nullptr;
+    int2 *tasks = nullptr;
+    int64_t *edge_off = nullptr;
+    int32_t *list = nullptr, *w_next = nullptr, *tie_list = nullptr, *tie_w = nullptr;
+  };
+
+  // Up to two pairs per resident warp the slowest pairs set the time of the band
+  // kernel, so those that fail go to the strips once their windows pass
+  // kBandHandLen rows (1,500 pairs of 1k..20k from w = 1,024: 63 -> 32 ms; more
+  // pairs keep the chip busy with narrower work: 8,000 pairs 81 ms, handed over
+  // 117).
+  bool few_pairs() const { return npairs <= 2 * (int64_t)c.nsm * std::max(blocks_per_sm_kz(), 1) * kKcWarps; }
+
+  // Workspace, sized for every pair; without it every pair stays on the band kernel.
+  int full_setup(Full &f) {
+    int64_t strips[kKxWidths];
+    for (int w = 0; w < kKxWidths; ++w) strips[w] = sums.strips[w];
+    f.tile = kx_choose(GA_GLOBAL, false, longest, strips, c.nsm);
+    const int64_t W = 64 * kKxTileK[f.tile];
+    if (longest > W * kKxMaxStrips || sums.rows > (4ull << 30) / 8) return GA_OK;
+    f.cap = strips[kKxTileK[f.tile] / 4 - 1];
+    f.bytes = sizeof(KXPairState) * (size_t)npairs + 16 + 8 * (size_t)sums.rows;
+    f.zero = c.al.try_get<char>(f.bytes);
+    if (f.zero) f.tasks = c.al.try_get<int2>((size_t)f.cap);
+    if (f.tasks) f.edge_off = c.al.try_get<int64_t>((size_t)npairs);
+    if (f.edge_off) f.list = c.al.try_get<int32_t>((size_t)npairs);
+    if (f.list) f.w_next = c.al.try_get<int32_t>((size_t)npairs);
+    if (f.w_next) f.tie_list = c.al.try_get<int32_t>((size_t)npairs);
+    if (f.tie_list) f.tie_w = c.al.try_get<int32_t>((size_t)npairs);
+    f.on = f.tie_w != nullptr;
+    return GA_OK;
+  }
+
+  // Whether the full matrices of all pairs are the faster way, in cycles.  They
+  // take the strips of the longest pair or the whole work at 2,850 cells a cycle
+  // (5.9 TCUPS).  The band kernel takes the longest pair's iterations of the
+  // attempts up to kBandHandLen (or to a width of a sixteenth of its rows, where
+  // most pairs of up to 15 % divergence are accepted), 345 cycles each and 105 more
+  // per warp of a scheduler, or the first attempts' cells at 2,400 a cycle; and the
+  // pairs that fail hold about 0.55 of the cells.  GB300, ms, all full / first
+  // attempts / with the failed ones full: 600 pairs of 1k..20k from w = 1,024 15.9 /
+  // 8.6 / 18.6, 1,500 34 / 13 / 31.6; from w = 64 1,500 34 / 26 / 55.
+  bool full_first(int32_t default_w0, bool per_pair) const {
+    double full = 0;
+    int64_t one[kKxWidths];
+    for (int w = 0; w < kKxWidths; ++w) one[w] = (longest + kx_width(w) - 1) / kx_width(w);
+    kx_choose(GA_GLOBAL, false, longest, one, c.nsm, &full);
+    full = std::max(full, full_cells / 2850.0);
+    const double rows = max_rows, stages = (double)(longest / kBandStageCols);
+    // (widths given per pair: the average window, one attempt)
+    double len = per_pair ? first_cells / std::max(1.0, (double)sums.rows) : 2.0 * default_w0 + 16.0;
+    double iterations = 0;
+    for (;;) {
+      iterations += std::max(128.0, std::min(rows, len - 1008.0) + 1.0) * stages + rows;
+      if (per_pair || len >= rows / 8.0) break;
+      len = 2.0 * len;
+      if (len > kBandHandLen) break;
+    }
+    const double warps = std::min(3.0, (double)npairs / (4.0 * c.nsm));
+    const double band = std::max(iterations * (345.0 + 105.0 * warps), first_cells / 2400.0);
+    return (few_pairs() ? 0.45 * full : full) <= band;
+  }
+
+  // Exact scores of the listed pairs, then their doubling; ties run their attempt.
+  int full_run(Full &f, KCParams kc, const int32_t *list, const int32_t *range, const int32_t *w_next) {
+    KXParams k{};
+    k.q_codes = Q.codes;
+    k.t_codes = T.codes;
+    k.q_off = Q.off;
+    k.t_off = T.off;
+    k.sorted = list;
+    k.range = range;
+    k.tasks = f.tasks;
+    k.state = reinterpret_cast<KXPairState *>(f.zero);
+    k.counter = reinterpret_cast<int32_t *>(f.zero + sizeof(KXPairState) * (size_t)npairs);
+    k.ntasks_dev = k.counter + 1;
+    k.edge_off = f.edge_off;
+    k.edges = reinterpret_cast<unsigned long long *>(f.zero + sizeof(KXPairState) * (size_t)npairs + 16);
+    k.scores = kc.scores;
+    k.status = &c.small->status;
+    std::memcpy(k.tables, c.sc.tables, sizeof(k.tables));
+    std::memcpy(k.sigma, c.sc.mat, sizeof(k.sigma));
+    k.A = c.sc.A;
+    k.alpha = c.sc.alpha;
+    k.beta = c.sc.beta;
+    KXTaskParams kt{};
+    kt.q_off = Q.off;
+    kt.t_off = T.off;
+    kt.sorted = list;
+    kt.range = range;
+    kt.W = 64 * kKxTileK[f.tile];
+    kt.tasks = f.tasks;
+    kt.edge_off = f.edge_off;
+    kt.ntasks = k.counter + 1;
+    if (cudaMemsetAsync(f.zero, 0, f.bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
+    kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
+    int occ = 0;
+    if (launch_kx(GA_GLOBAL, f.tile, k, 0, c.s, &occ) != cudaSuccess) return GA_ERR_CUDA;
+    const int kgrid = (int)std::min<int64_t>((f.cap + kKxWarps - 1) / kKxWarps, (int64_t)c.nsm * std::max(occ, 1));
+    c.dp_begin();
+    cudaError_t e = launch_kx(GA_GLOBAL, f.tile, k, kgrid, c.s);
+    c.dp_end();
+    if (e != cudaSuccess) return GA_ERR_CUDA;
+    BandVerdictParams v{};
+    v.q_off = Q.off;
+    v.t_off = T.off;
+    v.list = list;
+    v.range = range;
+    v.w_next = w_next;
+    v.w0 = kc.w0;
+    v.default_w0 = kc.default_w0;
+    v.alpha = kc.alpha;
+    v.beta = kc.beta;
+    v.sigma_max_pos = kc.sigma_max_pos;
+    v.scores = kc.scores;
+    v.w_used = kc.w_used;
+    v.retries = kc.retries;
+    v.cells = kc.cells;
+    v.tie_list = f.tie_list;
+    v.tie_count = &c.small->tie_range[1];
+    v.tie_w = f.tie_w;
+    if (launch_band_verdict(v, (int)std::min<int64_t>((npairs + kKcWarps - 1) / kKcWarps, 4 * (int64_t)c.nsm), c.s) !=
+        cudaSuccess)
+      return GA_ERR_CUDA;
+    kc.order = f.tie_list;
+    kc.range = c.small->tie_range;
+    kc.task_counter = &c.small->counters[launches++];
+    kc.w0 = f.tie_w;
+    kc.hand_count = nullptr;
+    c.dp_begin();
+    e = launch_kz(kc, grid, c.s);
+    c.dp_end();
+    c.launches += 2;
     return e == cudaSuccess ? GA_OK : GA_ERR_CUDA;
   }
 

@@ -527,6 +527,16 @@ __global__ void __launch_bounds__(128, 3) kz_kernel(const __grid_constant__ KCPa
       w = (w == 0) ? 1 : 2 * w;
       ++tries;
       __syncwarp();
+      if (p.hand_count) {
+        const int len = ::min(m, 2 * w + (dn < 0 ? -dn : dn) + K);
+        if (len > p.hand_len) {
+          if (t == 0) {
+            p.hand_list[atomicAdd(p.hand_count, 1)] = pid;
+            p.hand_w[pid] = w;
+          }
+          break;
+        }
+      }
     }
     unsigned long long c64 = *cells;
 #pragma unroll

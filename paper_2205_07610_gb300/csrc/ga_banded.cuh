@@ -52,6 +52,14 @@ struct KCParams {
   // lo == hi are skipped and nothing else is written.
   int32_t *bis_lo;
   int32_t *bis_hi;
+  // Doubling in kz_kernel: a pair whose attempt failed is not tried again but
+  // appended to hand_list (its next half-width in hand_w[pair]) once its windows
+  // would be longer than hand_len rows; the caller decides it by its exact score.
+  // null: never.
+  int32_t *hand_count;
+  int32_t *hand_list;
+  int32_t *hand_w;
+  int32_t hand_len;
 };
 
 __device__ __forceinline__ int64_t band_ub(int64_t m, int64_t n, int64_t smax, int64_t alpha,

@@ -19,7 +19,7 @@ constexpr Step kSteps[4][kKxTiles] = {
 constexpr int kLag = 115;  // rows a strip runs behind its left neighbour
 }  // namespace
 
-int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, int nsm) {
+int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, int nsm, double *cycles) {
   const Step *tab = kSteps[(profile ? 2 : 0) + (mode == 2 ? 1 : 0)];
   const int64_t sched = 4 * (int64_t)nsm;
   int best = -1;
@@ -34,6 +34,7 @@ int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, in
       tbest = t;
     }
   }
+  if (cycles) *cycles = tbest;
   return best;
 }
 

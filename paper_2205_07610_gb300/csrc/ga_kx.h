@@ -26,7 +26,8 @@ constexpr int kKxTileK[kKxTiles] = {4, 8, 12, 16, 20, 8, 16};
 // ceil(strips / schedulers) warps.  A lone warp's step is a latency, several
 // warps' the issue of their columns; both grow with K, the lag falls with it.
 // Measured on GB300 (cycles per row at one warp, and more per further one).
-int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, int nsm);
+// *cycles (nullable): the estimate.
+int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, int nsm, double *cycles = nullptr);
 
 // One launch of a mode's strip kernel, or (occ != null) its blocks per SM.
 cudaError_t launch_kx_local(int tile, const KXParams &p, int grid, cudaStream_t s, int *occ);

@@ -94,6 +94,9 @@ int blocks_per_sm_kc();
 // its edge buffer holds one KZEdge (16 bytes) per row and warp.
 cudaError_t launch_kz(const KCParams &p, int grid, cudaStream_t s);
 int blocks_per_sm_kz();
+// The doubling of pairs whose exact score is known (ga_bandfull.cuh).
+struct BandVerdictParams;
+cudaError_t launch_band_verdict(const BandVerdictParams &p, int grid, cudaStream_t s);
 
 // Launch / occupancy of tile `bin` (compile-time recursion over the tiles).
 template <class CELL, int MODE, int I = 0>

@@ -221,6 +221,26 @@ __device__ __forceinline__ int global_gap(int alpha, int beta, int64_t len) {
   return len == 0 ? 0 : -(int)(alpha + beta * (len - 1));
 }
 
+// Adds the pairs of a warp (shorter and longer sequence; 0: none) to the sizes of
+// a strip launch.
+__device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongSums *sums, int32_t *longest) {
+  const unsigned cmax = __reduce_max_sync(0xffffffffu, (unsigned)long_len);
+  // 32 x (2^30 + 1) needs more than 32 bits
+  unsigned long long rows = long_len ? (unsigned long long)short_len + 1 : 0;
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, off);
+  unsigned strips[kKxWidths];
+#pragma unroll
+  for (int w = 0; w < kKxWidths; ++w)
+    strips[w] = __reduce_add_sync(0xffffffffu, ((unsigned)long_len + kx_width(w) - 1) / kx_width(w));
+  if ((threadIdx.x & 31) == 0 && cmax) {
+    atomicMax(longest, (int)cmax);
+    atomicAdd(&sums->rows, rows);
+#pragma unroll
+    for (int w = 0; w < kKxWidths; ++w) atomicAdd(&sums->strips[w], (int)strips[w]);
+  }
+}
+
 // One pair (batch) or (query, target) combination (cross chunk).
 __device__ __forceinline__ void plan_one(const PlanParams &p, int64_t i, unsigned long long &my_cells,
                                          int &long_rows, int &long_cols) {
@@ -298,23 +318,7 @@ __global__ void plan_kernel(PlanParams p) {
   unsigned long long my_cells = 0;
   int long_rows = 0, long_cols = 0;
   if (i < p.npairs) plan_one(p, i, my_cells, long_rows, long_cols);
-  if (__any_sync(0xffffffffu, long_cols != 0)) {
-    const unsigned cmax = __reduce_max_sync(0xffffffffu, (unsigned)long_cols);
-    // 32 x (2^30 + 1) needs more than 32 bits
-    unsigned long long rows = long_cols ? (unsigned long long)long_rows + 1 : 0;
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, off);
-    unsigned strips[kKxWidths];
-#pragma unroll
-    for (int w = 0; w < kKxWidths; ++w)
-      strips[w] = __reduce_add_sync(0xffffffffu, ((unsigned)long_cols + kx_width(w) - 1) / kx_width(w));
-    if ((threadIdx.x & 31) == 0) {
-      atomicMax(p.rmax_long, (int)cmax);
-      atomicAdd(&p.long_sums->rows, rows);
-#pragma unroll
-      for (int w = 0; w < kKxWidths; ++w) atomicAdd(&p.long_sums->strips[w], (int)strips[w]);
-    }
-  }
+  if (__any_sync(0xffffffffu, long_cols != 0)) add_long_sums(long_rows, long_cols, p.long_sums, p.rmax_long);
   // one atomic per warp for the cell count
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) my_cells += __shfl_xor_sync(0xffffffffu, my_cells, off);
@@ -337,14 +341,18 @@ struct BandPlanParams {
   uint32_t *keys;
   int32_t *status;
   unsigned long long *cells;
-  int32_t *max_rows;
+  LongSums *sums;          // strips of the full matrices over the pairs to run
+  unsigned long long *est; // sum of rows times the first attempt's window length
+  int32_t *max_rows;       // longest query
+  int32_t *max_len;        // longest sequence
   int32_t *max_span;   // max of max(m + 1, 128) x super-stages + m, saturated
   int32_t stage_cols;  // columns of a super-stage of the packed band kernel
 };
 
 __global__ void band_plan_kernel(BandPlanParams p) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long my_cells = 0;
+  unsigned long long my_cells = 0, my_est = 0;
+  int short_len = 0, long_len = 0;
   if (i < p.npairs) {
     const int64_t m = p.q_off[i + 1] - p.q_off[i], n = p.t_off[i + 1] - p.t_off[i];
     int w = p.w0 ? p.w0[i] : p.default_w0;
@@ -364,6 +372,8 @@ __global__ void band_plan_kernel(BandPlanParams p) {
       if (p.w_used) p.w_used[i] = w;
     } else {
       my_cells = (unsigned long long)(m * n);
+      short_len = (int)(m < n ? m : n);
+      long_len = (int)(m < n ? n : m);
       atomicMax(p.max_rows, (int)m);
       {
         // bound on the packed band kernel's iteration numbers: its super-
@@ -379,15 +389,23 @@ __global__ void band_plan_kernel(BandPlanParams p) {
       const int64_t d = n - m;
       const int64_t nst = (n + p.stage_cols - 1) / p.stage_cols;
       const int64_t L = (d < 0 ? -d : d) + 2 * (int64_t)w + 16;
+      my_est = (unsigned long long)(m * (L < n ? L : n));
       const int lg = 63 - __clzll((long long)L);
       const int lb = ::min(63, lg * 4 + (int)((L >> (lg - 2)) & 3));
       key = (uint32_t)(kRBuckets - 1 - (int)((nst < 31 ? nst : 31) * 64 + lb));
     }
     p.keys[i] = key;
   }
+  add_long_sums(short_len, long_len, p.sums, p.max_len);
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) my_cells += __shfl_xor_sync(0xffffffffu, my_cells, off);
-  if ((threadIdx.x & 31) == 0 && my_cells) atomicAdd(p.cells, my_cells);
+  for (int off = 16; off >= 1; off >>= 1) {
+    my_cells += __shfl_xor_sync(0xffffffffu, my_cells, off);
+    my_est += __shfl_xor_sync(0xffffffffu, my_est, off);
+  }
+  if ((threadIdx.x & 31) == 0 && my_cells) {
+    atomicAdd(p.cells, my_cells);
+    atomicAdd(p.est, my_est);
+  }
 }
 
 __global__ void hist_kernel(const uint32_t *keys, int64_t n, int32_t *hist) {

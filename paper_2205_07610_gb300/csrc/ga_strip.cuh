@@ -81,6 +81,7 @@ struct KXParams {
   const int32_t *range;
   const int2 *tasks;             // (list entry, strip)
   int32_t ntasks;
+  const int32_t *ntasks_dev;     // the count on the device instead (nullable)
   const int64_t *edge_off;       // per list entry: its first edge word
   unsigned long long *edges;     // zeroed before the launch
   KXPairState *state;            // per list entry
@@ -503,11 +504,12 @@ __global__ void __launch_bounds__(32 * kKxWarps, 1) kx_kernel(const __grid_const
     }
     __syncthreads();
   }
+  const int ntasks = p.ntasks_dev ? *p.ntasks_dev : p.ntasks;
   for (;;) {
     int task = 0;
     if (t == 0) task = atomicAdd(p.counter, 1);
     task = __shfl_sync(0xffffffffu, task, 0);
-    if (task >= p.ntasks) break;
+    if (task >= ntasks) break;
     int li = 0, s = task, m = p.m, n = p.n, pid = 0;
     int64_t qs = 0, ts = 0, eo = 0;
     if (p.tasks) {

@@ -12,6 +12,7 @@ struct KXTaskParams {
   int32_t W;            // columns of a strip
   int2 *tasks;
   int64_t *edge_off;    // per list entry
+  int32_t *ntasks;      // their number (nullable)
 };
 
 // One block: every strip of every listed pair, the strips with the most strips
@@ -50,6 +51,7 @@ __global__ void kx_tasks_kernel(const __grid_constant__ KXTaskParams p) {
       start[k] = at;
       at += at_least;
     }
+    if (p.ntasks) *p.ntasks = at;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
