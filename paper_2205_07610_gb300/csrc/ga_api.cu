@@ -1435,39 +1435,39 @@ int features_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t
 // by length (columns per lane K = 8, 16, 24 or 32; longer queries run in
 // stages of 512 columns), flagged pairs recomputed exactly in int32.
 template <int K>
-int launch_kp(Call &c, KPParams &kp, int64_t max_grid) {
+int kp_grid(Call &c, const KPParams &kp) {
   const size_t smem = sizeof(uint32_t) * (size_t)kp_prof_words<K>(c.sc.A);
-  if (cudaFuncSetAttribute(kp_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return GA_ERR_CUDA;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp_kernel<K>, 32 * kKpWarps, smem) != cudaSuccess)
-    return GA_ERR_CUDA;
+  if (cudaFuncSetAttribute(kp_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp_kernel<K>, 32 * kKpWarps, smem) != cudaSuccess)
+    return 0;
   const int64_t ntasks = (int64_t)((kp.nqb + 1) / 2) * ((kp.ntv + kKpGroups - 1) / kKpGroups);
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>({ntasks, (int64_t)c.nsm * std::max(occ, 1), max_grid}));
-  c.dp_begin();
-  kp_kernel<K><<<grid, 32 * kKpWarps, smem, c.s>>>(kp);
-  c.dp_end();
-  return cudaGetLastError() == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(ntasks, (int64_t)c.nsm * std::max(occ, 1)));
+}
+
+template <int K>
+cudaError_t launch_kp(Call &c, const KPParams &kp, int grid, cudaStream_t s) {
+  kp_kernel<K><<<grid, 32 * kKpWarps, sizeof(uint32_t) * (size_t)kp_prof_words<K>(c.sc.A), s>>>(kp);
+  return cudaGetLastError();
 }
 
 // Tiles of the protein search: columns per lane K (16K columns per group)
-// and the measured relative rate of the kernel per computed cell on GB300
-// (wider tiles amortise the per-row work over more columns); a query of
-// several stages pays for its profile rebuilds and stage edges.
-constexpr int kKpTiles = 6;
-constexpr int kKpTileK[kKpTiles] = {8, 16, 20, 24, 28, 32};
-constexpr double kKpRate[kKpTiles] = {0.81, 0.92, 0.96, 1.0, 1.08, 1.02};
-constexpr double kKpStagedRate = 0.97;
+// and the measured cycles of a scheduler per column register and row on GB300
+// (wider tiles spread the per-row work over more columns); a query of several
+// stages pays 1 % for its profile rebuilds and stage edges.
+constexpr int kKpTiles = 7;
+constexpr int kKpTileK[kKpTiles] = {8, 12, 16, 20, 24, 28, 32};
+constexpr double kKpCycles[kKpTiles] = {12.3, 11.3, 10.8, 10.85, 10.45, 10.6, 10.65};
+constexpr double kKpStaged = 1.01;
 
-// Tile of a query of m columns: the one that minimises the estimated time
-// ceil(m / 16K) * 16K / rate(K).
+// Tile of a query of m columns: the one that minimises the estimated time.
 int kp_bin_for(int64_t m) {
   int best = kKpTiles - 1;
   double tbest = 1e300;
   for (int b = 0; b < kKpTiles; ++b) {
     const int64_t w = (int64_t)kKpG * kKpTileK[b];
     const int64_t nst = (m + w - 1) / w;
-    const double t = (double)(nst * w) / (kKpRate[b] * (nst > 1 ? kKpStagedRate : 1.0));
+    const double t = (double)(nst * w) * kKpCycles[b] * (nst > 1 ? kKpStaged : 1.0);
     if (t < tbest) {
       tbest = t;
       best = b;
@@ -1476,14 +1476,27 @@ int kp_bin_for(int64_t m) {
   return best;
 }
 
-int launch_kp_tile(Call &c, KPParams &kp, int64_t max_grid, int b) {
+int kp_grid_tile(Call &c, const KPParams &kp, int b) {
   switch (kKpTileK[b]) {
-    case 8: return launch_kp<8>(c, kp, max_grid);
-    case 16: return launch_kp<16>(c, kp, max_grid);
-    case 20: return launch_kp<20>(c, kp, max_grid);
-    case 24: return launch_kp<24>(c, kp, max_grid);
-    case 28: return launch_kp<28>(c, kp, max_grid);
-    default: return launch_kp<32>(c, kp, max_grid);
+    case 8: return kp_grid<8>(c, kp);
+    case 12: return kp_grid<12>(c, kp);
+    case 16: return kp_grid<16>(c, kp);
+    case 20: return kp_grid<20>(c, kp);
+    case 24: return kp_grid<24>(c, kp);
+    case 28: return kp_grid<28>(c, kp);
+    default: return kp_grid<32>(c, kp);
+  }
+}
+
+cudaError_t launch_kp_tile(Call &c, const KPParams &kp, int grid, int b, cudaStream_t s) {
+  switch (kKpTileK[b]) {
+    case 8: return launch_kp<8>(c, kp, grid, s);
+    case 12: return launch_kp<12>(c, kp, grid, s);
+    case 16: return launch_kp<16>(c, kp, grid, s);
+    case 20: return launch_kp<20>(c, kp, grid, s);
+    case 24: return launch_kp<24>(c, kp, grid, s);
+    case 28: return launch_kp<28>(c, kp, grid, s);
+    default: return launch_kp<32>(c, kp, grid, s);
   }
 }
 
@@ -1549,7 +1562,7 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
     std::stable_sort(b.begin(), b.end(), [&](int32_t x, int32_t y) {
       return hqo[(size_t)x + 1] - hqo[(size_t)x] > hqo[(size_t)y + 1] - hqo[(size_t)y];
     });
-  {
+  if (stats) {  // the cell count needs the valid targets' lengths
     std::vector<int64_t> hto((size_t)nt + 1);
     std::vector<uint8_t> htb((size_t)nt);
     if (cudaMemcpy(hto.data(), t_off, sizeof(int64_t) * (size_t)(nt + 1), cudaMemcpyDeviceToHost) != cudaSuccess ||
@@ -1566,11 +1579,6 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   if (!flat.empty() &&
       cudaMemcpyAsync(dq, flat.data(), sizeof(int32_t) * flat.size(), cudaMemcpyHostToDevice, c.s) != cudaSuccess)
     return GA_ERR_CUDA;
-  // per-group stage edges: every group slot of the largest grid
-  const int64_t max_grid = (int64_t)c.nsm * 4;
-  const int64_t stride = (int64_t)std::max(max_len, 0) + 64;
-  int2 *bnd = c.al.get<int2>((size_t)max_grid * kKpGroups * (size_t)stride);
-  if (c.al.failed) return GA_ERR_OOM;
   KPParams kp{};
   kp.q_codes = q_codes;
   kp.q_off = q_off;
@@ -1589,20 +1597,50 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   kp.rerun_list = rerun;
   kp.rerun_count = &c.small->rerun_range[1];
   kp.rerun_cap = rerun_cap;
-  kp.bnd = bnd;
-  kp.bnd_stride = stride;
-  size_t off = 0;
+  kp.bnd_stride = (int64_t)std::max(max_len, 0) + 64;
+  // One launch per bin, each on a side stream: the chip stays full over the ends of
+  // the launches, and a search of a few queries has all its bins in flight (8
+  // queries x 2,000 targets 4.65 ms in order, 1.9 together).  The bins whose rows cost most come
+  // first, so the last launch's longest target is a short chain.  Bins of several
+  // stages keep their edges in a buffer of their own; where these would take more
+  // than 4 GB the launches run in order and share one.
+  KPParams kps[kKpTiles];
+  int grids[kKpTiles] = {}, order[kKpTiles], nlaunch = 0;
+  size_t edges[kKpTiles] = {}, edge_sum = 0, edge_max = 0, off = 0;
+  double chain[kKpTiles] = {};
   for (int b = 0; b < kKpTiles; ++b) {
-    if (bins[b].empty() || ntv == 0) {
-      off += bins[b].size();
-      continue;
-    }
-    kp.queries = dq + off;
+    const int32_t *queries = dq + off;
+    off += bins[b].size();
+    if (bins[b].empty() || ntv == 0) continue;
+    kp.queries = queries;
     kp.nqb = (int32_t)bins[b].size();
     kp.task_counter = &c.small->counters[b];
-    off += bins[b].size();
-    rc = launch_kp_tile(c, kp, max_grid, b);
-    if (rc) return rc;
+    const int64_t W = (int64_t)kKpG * kKpTileK[b], nst = (hqo[(size_t)bins[b][0] + 1] - hqo[(size_t)bins[b][0]] + W - 1) / W;
+    if ((grids[b] = kp_grid_tile(c, kp, b)) <= 0) return GA_ERR_CUDA;
+    if (nst > 1) edges[b] = (size_t)grids[b] * kKpGroups * (size_t)kp.bnd_stride;
+    edge_sum += edges[b];
+    edge_max = std::max(edge_max, edges[b]);
+    chain[b] = (double)(nst * W);
+    kps[b] = kp;
+    order[nlaunch++] = b;
+  }
+  std::stable_sort(order, order + nlaunch, [&](int x, int y) { return chain[x] > chain[y]; });
+  const bool together = edge_sum * sizeof(int2) <= (4ull << 30);
+  int2 *bnd = edge_max ? c.al.get<int2>(together ? edge_sum : edge_max) : nullptr;
+  if (c.al.failed) return GA_ERR_OOM;
+  {
+    DpFork fk(c);
+    if ((rc = fk.begin(together ? nlaunch : 0))) return rc;
+    for (int i = 0; i < nlaunch; ++i) {
+      const int b = order[i];
+      kps[b].bnd = bnd;
+      if (together && bnd) bnd += edges[b];
+      const cudaStream_t ls = fk.launch_begin();
+      const cudaError_t e = launch_kp_tile(c, kps[b], grids[b], b, ls);
+      fk.launch_end();
+      if (e != cudaSuccess) return GA_ERR_CUDA;
+    }
+    if ((rc = fk.end())) return rc;
   }
   // exact int32 rerun of flagged pairs (rare: a local score near 32767).
   // Each pass reruns the pairs of the list; when the kernels flagged more

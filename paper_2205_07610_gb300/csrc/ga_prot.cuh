@@ -14,22 +14,25 @@
 // One profile per block, in shared memory, for the stage of 16K columns the
 // block is working on: the 4 warps (8 groups) of a block take 8 targets of
 // one query pair per task (targets sorted longest first, tasks
-// query-pair-major), and the block rebuilds the profile from a transposed
-// sigma table only when its query pair or stage changes.  A row then costs
+// target-major, so the longest chains start first and the last tasks are short),
+// and the block rebuilds the profile from a transposed sigma table when its
+// query pair or stage changes (2k cycles against 300k of a task).  A row then costs
 // K/4 16-byte shared loads per lane and no per-column byte permute.
 // Queries longer than 16K columns run in stages of 16K columns; lane 15
 // stores the right edge of a stage (packed H and outgoing F per row) to a
 // per-group global buffer, which the next stage reads back in batches of
 // 16 rows through shared memory for its lane 0.
 //
-// Padding: rows past a target's end use the all-zero profile row and
-// columns past a query's end have score 0; in local mode such cells never
-// exceed the largest real cell, so the running maximum is exact.  A pair
-// whose running maximum reaches 32767 - sigma_max is queued for an exact
-// int32 rerun: its score entry is set to kRerunMark (no real score comes
-// near it: every admitted score is below 2^30) and its id is appended to the
-// rerun list while the list has room, so the caller can always find every
-// flagged pair by scanning the scores when the list overflowed.
+// Padding: rows before a target's first and past its last use the all-zero
+// profile row and columns past a query's end have score 0.  A row before the
+// first leaves the boundary state (H = 0, E = F = -alpha) as it is, and in local
+// mode such cells never exceed the largest real cell, so the running maximum
+// is exact. A pair whose running maximum reaches 32767 - sigma_max is queued
+// for an exact int32 rerun: its score entry is set to kRerunMark (no real
+// score comes near it: every admitted score is below 2^30) and its id is
+// appended to the rerun list while the list has room, so the caller can
+// always find every flagged pair by scanning the scores when the list
+// overflowed.
 #pragma once
 
 #include "ga_dp.cuh"
@@ -74,13 +77,16 @@ __host__ __device__ constexpr int kp_prof_words(int A) {
   return (A + 1) * kKpG * K;
 }
 
-// Resident blocks per SM requested from ptxas: what shared memory allows for
-// BLOSUM-sized alphabets (24 symbols + pad: (A+1) x 16K words of profile per
-// block plus 3.7 KB of static tables and rings; 51.2 KB for K = 32, so 4
-// blocks fit in the SM's 228 KB).
+// Resident blocks per SM requested from ptxas.  The row loop is bound by the ALU
+// pipe: 3.5 instructions at 2 cycles a column and row (one 3-way max, two fused
+// add-maxes, half a max for the running maximum), 10.5..12.3 cycles measured with
+// the row's own work.  Registers for an unrolled loop without spills are worth
+// more than the last block: cycles a column on GB300, with as many blocks as shared
+// memory takes / as below, K = 8: 13.4 / 12.3, 12: 11.7 / 11.3, 16: 12.0 / 10.8,
+// 20: 11.7 / 10.9, 28: 10.8 / 10.6, 32: 10.9 / 10.7 (24: 10.5 with 4, 11.3 with 3).
 template <int K>
 struct KPMinBlocks {
-  static constexpr int value = K <= 8 ? 8 : K <= 16 ? 6 : K <= 20 ? 5 : 4;
+  static constexpr int value = K <= 8 ? 7 : K <= 16 ? 5 : K <= 24 ? 4 : 3;
 };
 
 template <int K>
@@ -105,7 +111,8 @@ __global__ void __launch_bounds__(32 * kKpWarps, KPMinBlocks<K>::value) kp_kerne
   }
   uint8_t *ring = ring_s[grp];
   uint2 *in_ring = in_ring_s[grp];
-  int2 *bnd = p.bnd + (size_t)(blockIdx.x * kKpGroups + grp) * (size_t)p.bnd_stride;
+  // rows -15 .. Rw of the stage edge of a group
+  int2 *bnd = p.bnd + (size_t)(blockIdx.x * kKpGroups + grp) * (size_t)p.bnd_stride + G;
   const int A = p.A, alpha = p.alpha, beta = p.beta;
   const T NB = Cell::splat(-beta), NAc = Cell::splat(-alpha);
   const int ngroups = (p.ntv + kKpGroups - 1) / kKpGroups;
@@ -119,7 +126,7 @@ __global__ void __launch_bounds__(32 * kKpWarps, KPMinBlocks<K>::value) kp_kerne
     __syncthreads();
     const int task = task_s;
     if ((int64_t)task >= ntasks) break;
-    const int qp = task / ngroups, tg = task % ngroups;
+    const int tg = task / nqp, qp = task - tg * nqp;
     int kq[2], m[2];
     int64_t qs[2];
 #pragma unroll
@@ -169,11 +176,11 @@ __global__ void __launch_bounds__(32 * kKpWarps, KPMinBlocks<K>::value) kp_kerne
         __syncthreads();
       }
       if (Rw == 0) continue;  // a warp past the last target
-      // ---- row codes, refilled G rows ahead -----------------------------
+      // ---- row codes, refilled G rows ahead; the pad code outside 1..len --
       auto fill_batch = [&](int b) {
         const int r = b * G + 1 + t;
         uint8_t c = (uint8_t)A;
-        if (r <= len) {
+        if ((unsigned)(r - 1) < (unsigned)len) {
           const unsigned x = (unsigned)(trem + r - 1), wq = x / 6u;
           c = (uint8_t)((__ldg(tword + wq) >> (5u * (x - 6u * wq))) & 31u);
         }
@@ -185,89 +192,93 @@ __global__ void __launch_bounds__(32 * kKpWarps, KPMinBlocks<K>::value) kp_kerne
       // loaded while lane 0 still reads batch b-1, and before lane 15
       // overwrites those rows with this stage's right edge (15 rows later)
       auto load_edge = [&](int b) {
-        if (s > 0) {
-          const int r = b * G + 1 + t;
-          if (r <= Rw) {
-            const int2 v = bnd[r];
-            in_ring[(r - 1) & (2 * G - 1)] = make_uint2((uint32_t)v.x, (uint32_t)v.y);
+        const int r = b * G + 1 + t;
+        uint2 v = make_uint2(Cell::splat(0), NAc);
+        if (r <= Rw) {
+          const int2 x = bnd[r];
+          v = make_uint2((uint32_t)x.x, (uint32_t)x.y);
+        }
+        in_ring[(r - 1) & (2 * G - 1)] = v;
+      };
+      const bool store_edge = s + 1 < nstage && t == G - 1;
+
+      // The rows of this stage; EDGE: the left inputs come from the stage before.
+      auto rows = [&](auto edge_tag) {
+        constexpr bool EDGE = decltype(edge_tag)::value;
+        __syncwarp();
+        fill_batch(-1);
+        fill_batch(0);
+        fill_batch(1);
+        if constexpr (EDGE) load_edge(0);
+        __syncwarp();
+        T H[K], E[K], w[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+          H[j] = Cell::splat(0);
+          E[j] = NAc;  // E(1, j) = H(0, j) - alpha
+        }
+        T Hdiag = Cell::splat(0), Hleft = Cell::splat(0), Fin = NAc;
+        if constexpr (EDGE) {
+          if (t == 0) {
+            Hleft = in_ring[0].x;
+            Fin = in_ring[0].y;
           }
         }
-      };
-      const bool edge_out = s + 1 < nstage;
-      __syncwarp();
-      fill_batch(0);
-      fill_batch(1);
-      load_edge(0);
-      __syncwarp();
-
-      T H[K], E[K];
-#pragma unroll
-      for (int j = 0; j < K; ++j) {
-        H[j] = Cell::splat(0);
-        E[j] = NAc;  // E(1, j) = H(0, j) - alpha
-      }
-      auto left = [&](int r, T &hl, T &fl) {  // lane 0: (H(r, 16Ks), F(r, 16Ks+1))
-        if (s == 0) {
-          hl = Cell::splat(0);
-          fl = NAc;
-        } else {
-          const uint2 v = in_ring[(r - 1) & (2 * G - 1)];
-          hl = v.x;
-          fl = v.y;
-        }
-      };
-      T Hdiag = Cell::splat(0), Hleft = Cell::splat(0), Fin = Cell::splat(CellInfo<Cell>::kNeg);
-      if (t == 0) left(1, Hleft, Fin);
-      const uint32_t *plane = kp_prof + t * 4;
-
-      // One row step of this lane.  GENERAL: some lane of the group is
-      // outside rows 1..Rw or lane 0's next edge row is past Rw; the other
-      // batches of G steps run without those checks.
-      const int nit = Rw + G - 1;
-      auto step = [&](int it, uint32_t rc, auto general_tag) {
-        constexpr bool GENERAL = decltype(general_tag)::value;
-        const int r = it - t + 1;
-        // lane 0's next left input, read before the row update
-        T hl = Cell::splat(0), fl = NAc;
-        if (t == 0 && (!GENERAL || it + 2 <= Rw)) left(it + 2, hl, fl);
-        T Hout = H[K - 1], Fout = Cell::splat(CellInfo<Cell>::kNeg);
-        if (!GENERAL || (unsigned)(r - 1) < (unsigned)Rw) {
-          const uint4 *pr = reinterpret_cast<const uint4 *>(plane + (size_t)rc * W);
-          uint32_t w[K];
+        const uint32_t *plane = kp_prof + t * 4;
+        auto load_row = [&](uint32_t rc) {
+          const uint4 *pr = reinterpret_cast<const uint4 *>(plane + rc * (uint32_t)W);
 #pragma unroll
           for (int q = 0; q < CH; ++q) {
             const uint4 a = pr[q * 16];
             w[4 * q] = a.x; w[4 * q + 1] = a.y; w[4 * q + 2] = a.z; w[4 * q + 3] = a.w;
           }
-          Fout = dp_row<Cell, kModeLocal, K>(
-              H, E, Hdiag, Fin, NB, best, [&](int j) -> T { return w[j]; }, [&](int) -> T { return NAc; });
-          Hout = H[K - 1];
-          if (t == G - 1 && edge_out) bnd[r] = make_int2((int)Hout, (int)Fout);
-        }
-        Hdiag = Hleft;
-        Hleft = __shfl_up_sync(0xffffffffu, Hout, 1, G);
-        Fin = __shfl_up_sync(0xffffffffu, Fout, 1, G);
-        if (t == 0) {
-          Hleft = hl;
-          Fin = fl;
-        }
-      };
-      for (int it0 = 0; it0 < nit; it0 += G) {
-        __syncwarp();
-        fill_batch(it0 / G + 2);
-        load_edge(it0 / G + 1);
-        __syncwarp();
-        // this lane's ring entries of the batch are contiguous (mirrored ring)
-        const uint8_t *rp = ring + ((it0 - t + 1) & (kRing - 1));
-        if (it0 >= G - 1 && it0 + G + 1 <= Rw) {
-#pragma unroll 2
-          for (int k = 0; k < G; ++k) step(it0 + k, rp[k], std::false_type{});
-        } else {
+        };
+        uint32_t rc = ring[(1 - t) & (kRing - 1)];  // code of the next row
+        const int nit = Rw + G - 1;
+        for (int it0 = 0; it0 < nit; it0 += G) {
+          __syncwarp();
+          fill_batch(it0 / G + 2);
+          if constexpr (EDGE) load_edge(it0 / G + 1);
+          __syncwarp();
+          // this lane's ring entries of the batch, from its second row, are contiguous
+          // (mirrored ring)
+          const uint8_t *rp = ring + ((it0 - t + 2) & (kRing - 1));
+          const uint2 *ir = in_ring + ((it0 + 1) & (2 * G - 1));  // (it0 + k + 1: wraps at k = 15)
+          int2 *bw = bnd + (it0 - t + 1);
           const int nb = ::min(G, nit - it0);
-          for (int k = 0; k < nb; ++k) step(it0 + k, rp[k], std::true_type{});
+#pragma unroll 4
+          for (int k = 0; k < nb; ++k) {
+            load_row(rc);
+            rc = rp[k];
+            // lane 0's next left input, read before the row update
+            uint2 left = make_uint2(Cell::splat(0), NAc);
+            if constexpr (EDGE) left = k == G - 1 ? in_ring[(it0 + G) & (2 * G - 1)] : ir[k];
+#pragma unroll
+            for (int j = K - 1; j >= 1; --j) H[j] = Cell::add(H[j - 1], w[j]);
+            H[0] = Cell::add(Hdiag, w[0]);
+            T F = Fin;
+#pragma unroll
+            for (int j = 0; j < K; ++j) {
+              H[j] = Cell::max3_relu(H[j], E[j], F);
+              const T X = Cell::add(H[j], NAc);
+              E[j] = Cell::addmax(E[j], NB, X);
+              F = Cell::addmax(F, NB, X);
+              if ((j & 1) == 1) best = Cell::max3(best, H[j - 1], H[j]);
+            }
+            if (store_edge) bw[k] = make_int2((int)H[K - 1], (int)F);
+            Hdiag = Hleft;
+            Hleft = __shfl_up_sync(0xffffffffu, H[K - 1], 1, G);
+            Fin = __shfl_up_sync(0xffffffffu, F, 1, G);
+            if (t == 0) {
+              Hleft = left.x;
+              Fin = left.y;
+            }
+          }
         }
-      }
-      __syncwarp();  // the edge stores are ordered before the next stage's loads
+        __syncwarp();  // the edge stores are ordered before the next stage's loads
+      };
+      if (s == 0) rows(std::false_type{});
+      else rows(std::true_type{});
     }
 
     // ---- scores ----------------------------------------------------------

@@ -1,0 +1,46 @@
+"""GPU: the protein search kernel (ga_prot.cuh) at the edges of its tiles, stages and
+row batches, for alphabets and gap costs at the ends of their ranges."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+import paper_2205_07610_gb300 as ga  # noqa: E402
+
+NTHREADS = os.cpu_count() or 8
+WIDTHS = [128, 192, 256, 320, 384, 448, 512, 640, 768, 896, 1024]
+
+
+@pytest.mark.parametrize("A,alpha,beta,lo,hi", [(20, 11, 1, -4, 11), (5, 1, 1, -1, 1), (31, 4096, 4096, -127, 127),
+                                                (24, 1, 1, -2, 9)])
+def test_tile_stage_and_batch_edges(A, alpha, beta, lo, hi):
+    rng = np.random.default_rng(A)
+    mat = rng.integers(lo, 1, size=(A, A)).astype(np.int8)
+    np.fill_diagonal(mat, hi)
+    qlens = [0, 1, 2] + [w + d for w in WIDTHS for d in (-1, 0, 1)]
+    qs = [rng.integers(0, A, size=n).astype(np.uint8) for n in qlens]
+    ts = [rng.integers(0, A, size=n).astype(np.uint8) for n in
+          [0, 1, 2, 14, 15, 16, 17, 18, 30, 31, 32, 33, 47, 48, 49, 63, 64, 65, 130]]
+    # related targets: alignments that cross stage edges and end in the last rows and columns
+    for k in range(8, len(qs), 3):
+        t = np.delete(qs[k], rng.integers(0, len(qs[k]), size=len(qs[k]) // 30))
+        ts += [t, t[-int(rng.integers(20, 60)):]]
+    qc, qo = synth.pack_csr(qs)
+    tc, to = synth.pack_csr(ts)
+    dev = [torch.from_numpy(a).cuda() for a in (qc, qo, tc, to)]
+    got, st = ga.align_cross(*dev, mat, alpha, beta, "local", stats=True)
+    want, _ = oracle.cross(qc, qo, tc, to, mat, alpha, beta, "local", nthreads=NTHREADS)
+    assert np.array_equal(got.cpu().numpy().ravel(), want.ravel()) and st["status"] == 0
+    # one query, so that its bin is the only launch; the same scores
+    for k in (1, 12, len(qs) - 1):
+        one = ga.align_cross(dev[0], dev[1][k:k + 2].contiguous(), *dev[2:], mat, alpha, beta, "local")
+        assert torch.equal(one.ravel(), got[k])
