@@ -1500,6 +1500,136 @@ cudaError_t launch_kp_tile(Call &c, const KPParams &kp, int grid, int b, cudaStr
   }
 }
 
+// Longest targets of a search that go to the strip kernels (ga_strip.cuh).  In the
+// search kernel a target's rows follow one another through the stages of a query:
+// 2,000 rows of a 900-residue query take a millisecond however few the targets are.
+// Strips spread such a pair over many warps at about a third of the search kernel's
+// rate, so they take the targets whose chains would outlast the rest of the work.
+struct KpSplit {
+  int ntargets = 0;
+  int tile = 0;
+  int64_t npairs = 0, strips = 0, rows = 0, grid = 0;
+  KXParams kx{};
+};
+
+// Chooses the number of targets, in cycles: strips as estimated by kx_choose and
+// 30k and 8 a pair for their task list, then the search kernel's remaining work and
+// twice its longest remaining chain (its launches start one after another once the
+// chip is full), as sides of a right angle; 3 % less than no split or none.  GB300,
+// ms, search kernel alone / so split: 4 queries x 500 targets 1.53 / 0.56, 8 x 2,000
+// 1.92 / 1.2, 16 x 2,000 2.6 / 1.9, 40 x 500 3.05 / 1.96, 90 x 500 3.4 / 2.25, 8 x
+// 8,000 2.85 / 2.58; with 64 targets split off 90 x 2,000 6.2 / 6.5, 90 x 8,000 22.0
+// / 22.8 (left alone).
+void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascending */, const KPTop &top,
+                     int64_t max_len, KpSplit &sp) {
+  const size_t nq = qlen.size();
+  if (nq == 0 || qlen[0] == 0 || std::max(c.sc.smax, 0) + c.sc.alpha > kKxMaxStep) return;
+  // pairs that may leave 16 bits stay with the search kernel, which counts them
+  if (std::min(qlen[nq - 1], max_len) * std::max(c.sc.smax, 0) >= 32767 - c.sc.smax) return;
+  // per unit of target rows: cycles of a warp over all query pairs (two targets a
+  // warp), and the slowest row of one
+  double work = 0, lone = 0, full = 0;
+  for (size_t k = 0; k < nq; ++k) {
+    const int b = kp_bin_for(qlen[k]), K = kKpTileK[b];
+    const double nst = (double)((qlen[k] + kKpG * K - 1) / (kKpG * K));
+    work += nst * K * kKpCycles[b] / 4.0;
+    lone = std::max(lone, nst * (75.0 + 15.2 * K));
+    full = std::max(full, nst * K * kKpCycles[b]);
+  }
+  const double sched = 4.0 * c.nsm;
+  std::vector<int64_t> above[kKxWidths], below(nq + 1, 0);  // strips of queries k.. / residues of queries ..k
+  for (size_t k = 0; k < nq; ++k) below[k + 1] = below[k] + qlen[k];
+  for (int w = 0; w < kKxWidths; ++w) {
+    above[w].assign(nq + 1, 0);
+    for (size_t k = nq; k-- > 0;) above[w][k] = above[w][k + 1] + (qlen[k] + kx_width(w) - 1) / kx_width(w);
+  }
+  int64_t strips[kKxWidths] = {}, rows = 0;
+  double rest = (double)top.residues, best = 0;
+  const int64_t longest = std::max(qlen[nq - 1], max_len);
+  for (int r = 0; r <= kKpTop; ++r) {
+    const int64_t n = r < kKpTop ? top.target[r].y : 0;
+    if (n < 0 || r == kKpTop || r % 8 == 0) {
+      double kx = 0;
+      int tile = 0;
+      if (r > 0) {
+        tile = kx_choose(GA_LOCAL, true, longest, strips, c.nsm, &kx);
+        kx += 30e3 + 8.0 * r * nq;
+        if (longest > 64 * kKxTileK[tile] * kKxMaxStrips || rows > (1ll << 30) / 8) return;
+      }
+      const bool none_left = n < 0 || (r < kKpTop && n == 0);
+      const double warps = std::min(3.0, std::max(1.0, rest * nq / 4.0 / std::max<int64_t>(n, 1) / sched));
+      const double kp = none_left ? 0 : std::hypot(rest * work / sched, 2.0 * n * std::max(lone, full * warps));
+      if (r == 0 || kx + kp < best) {
+        best = r == 0 ? 0.97 * kp : kx + kp;
+        sp.ntargets = r;
+        sp.tile = tile;
+        sp.npairs = (int64_t)r * (int64_t)nq;
+        sp.strips = r ? strips[kKxTileK[tile] / 4 - 1] : 0;
+        sp.rows = rows;
+      }
+      if (none_left || r == kKpTop) return;
+    }
+    const size_t k = std::upper_bound(qlen.begin(), qlen.end(), n) - qlen.begin();  // queries up to n residues
+    for (int w = 0; w < kKxWidths; ++w) strips[w] += (int64_t)k * ((n + kx_width(w) - 1) / kx_width(w)) + above[w][k];
+    rows += below[k] + (int64_t)(nq - k) * n + (int64_t)nq;
+    rest -= (double)n;
+  }
+}
+
+// Task list and workspace of the chosen targets, on the call's stream; without the
+// workspace the search kernel keeps them.
+int kp_split_prepare(Call &c, const SetView &Q, const SetView &T, int64_t nt, const int32_t *queries, int64_t nqv,
+                     const int32_t *sorted, int32_t *scores, KpSplit &sp) {
+  const size_t head = sizeof(KXPairState) * (size_t)sp.npairs + 16, bytes = head + 8 * (size_t)sp.rows;
+  char *zero = c.al.try_get<char>(bytes);
+  int2 *tasks = zero ? c.al.try_get<int2>((size_t)sp.strips) : nullptr;
+  int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)sp.npairs) : nullptr;
+  int32_t *list = edge_off ? c.al.try_get<int32_t>((size_t)sp.npairs) : nullptr;
+  if (!list) {
+    sp.ntargets = 0;
+    return GA_OK;
+  }
+  KXParams &k = sp.kx;
+  k.q_codes = Q.codes;
+  k.t_codes = T.codes;
+  k.q_off = Q.off;
+  k.t_off = T.off;
+  k.sorted = list;
+  k.range = c.small->hand_range;
+  k.tasks = tasks;
+  k.ntasks = (int32_t)sp.strips;
+  k.state = reinterpret_cast<KXPairState *>(zero);
+  k.counter = reinterpret_cast<int32_t *>(zero + sizeof(KXPairState) * (size_t)sp.npairs);
+  k.edge_off = edge_off;
+  k.edges = reinterpret_cast<unsigned long long *>(zero + head);
+  k.scores = scores;
+  k.status = &c.small->status;
+  k.nt = nt;
+  std::memcpy(k.sigma, c.sc.mat, sizeof(k.sigma));
+  k.A = c.sc.A;
+  k.alpha = c.sc.alpha;
+  k.beta = c.sc.beta;
+  int occ = 0;
+  if (launch_kx(GA_LOCAL, sp.tile, k, 0, c.s, &occ) != cudaSuccess) return GA_ERR_CUDA;
+  sp.grid = std::min<int64_t>((sp.strips + kKxWarps - 1) / kKxWarps, (int64_t)c.nsm * std::max(occ, 1));
+  kp_split_pairs_kernel<<<(unsigned)((sp.npairs + 255) / 256), 256, 0, c.s>>>(queries, (int32_t)nqv, sorted, nt,
+                                                                              (int32_t)sp.npairs, list,
+                                                                              c.small->hand_range);
+  KXTaskParams kt{};
+  kt.q_off = Q.off;
+  kt.t_off = T.off;
+  kt.sorted = list;
+  kt.range = k.range;
+  kt.nt = nt;
+  kt.W = 64 * kKxTileK[sp.tile];
+  kt.tasks = tasks;
+  kt.edge_off = edge_off;
+  if (cudaMemsetAsync(zero, 0, bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
+  kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
+  c.launches += 2;
+  return cudaGetLastError() == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+}
+
 int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, int64_t nq,
                         const uint8_t *t_codes, const int64_t *t_off, int64_t nt, int32_t *scores,
                         ga_stats *stats, cudaEvent_t e0, cudaEvent_t e1) {
@@ -1526,19 +1656,24 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   scan_partials_kernel<<<kScanTiles, kScanTile, 0, c.s>>>(c.hist, c.small->scan_partials);
   scan_apply_kernel<<<kScanTiles, kScanTile, 0, c.s>>>(c.hist, c.small->scan_partials, c.cursor, c.small->ranges);
   scatter_kernel<<<nbt, 256, 0, c.s>>>(keys, nt, c.cursor, sorted);
-  c.launches += 5;
+  KPTop *dtop = c.al.get<KPTop>(1);
+  if (c.al.failed) return GA_ERR_OOM;
+  kp_top_kernel<<<kKpTop / 256, 256, 0, c.s>>>(t_off, nt, sorted, c.small->ranges, dtop);
+  c.launches += 6;
   if (cudaGetLastError() != cudaSuccess) return GA_ERR_CUDA;
-  // host view: query offsets and validity, target count and longest target
+  // host view: query offsets and validity, target count, longest targets
+  std::vector<KPTop> top(1);
   std::vector<int64_t> hqo((size_t)nq + 1);
   std::vector<uint8_t> hqb((size_t)nq);
   Small *hs = (Small *)pinned_scratch();
   static_assert(sizeof(Small) <= 8192, "pinned scratch holds the call's scalars");
   if (cudaMemcpyAsync(hqo.data(), q_off, sizeof(int64_t) * (size_t)(nq + 1), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
       cudaMemcpyAsync(hqb.data(), Q.bad, (size_t)nq, cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
+      cudaMemcpyAsync(top.data(), dtop, sizeof(KPTop), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
       cudaMemcpyAsync(hs, c.small, sizeof(Small), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
       cudaStreamSynchronize(c.s) != cudaSuccess)
     return GA_ERR_CUDA;
-  const int32_t ntv = hs->ranges[1] - hs->ranges[0];
+  int32_t ntv = hs->ranges[1] - hs->ranges[0];
   const int32_t max_len = hs->max_rows;
   bool any_bad = ntv < nt;
   for (int64_t k = 0; k < nq; ++k) any_bad |= hqb[k] != 0;
@@ -1549,11 +1684,13 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   }
   // query bins: one tile per query (kp_bin_for)
   std::vector<int32_t> bins[kKpTiles];
+  std::vector<int64_t> qlen;
   int64_t cells = 0, tcells = 0;
   for (int64_t k = 0; k < nq; ++k) {
     if (hqb[k]) continue;
     const int64_t m = hqo[k + 1] - hqo[k];
     bins[kp_bin_for(m)].push_back((int32_t)k);
+    qlen.push_back(m);
     cells += m;
   }
   // the kernel packs queries 2i and 2i+1 of a bin into one register; sorted
@@ -1579,13 +1716,23 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   if (!flat.empty() &&
       cudaMemcpyAsync(dq, flat.data(), sizeof(int32_t) * flat.size(), cudaMemcpyHostToDevice, c.s) != cudaSuccess)
     return GA_ERR_CUDA;
+  const int32_t ntv_all = ntv;
+  KpSplit sp;
+  if (ntv > 0) {
+    std::sort(qlen.begin(), qlen.end());
+    kp_split_choose(c, qlen, top[0], max_len, sp);
+    if (sp.ntargets &&
+        (rc = kp_split_prepare(c, Q, T, nt, dq, (int64_t)flat.size(), sorted, scores, sp)))
+      return rc;
+    ntv -= sp.ntargets;
+  }
   KPParams kp{};
   kp.q_codes = q_codes;
   kp.q_off = q_off;
   kp.t_codes = t_codes;
   kp.t_packed5 = t_packed5;
   kp.t_off = t_off;
-  kp.t_sorted = sorted;
+  kp.t_sorted = sorted + sp.ntargets;
   kp.ntv = ntv;
   kp.nt = nt;
   kp.A = c.sc.A;
@@ -1630,7 +1777,14 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   if (c.al.failed) return GA_ERR_OOM;
   {
     DpFork fk(c);
-    if ((rc = fk.begin(together ? nlaunch : 0))) return rc;
+    const int nkx = sp.ntargets > 0;
+    if ((rc = fk.begin(together || nlaunch == 1 ? nlaunch + nkx : 0))) return rc;
+    if (nkx) {
+      const cudaStream_t ls = fk.launch_begin();
+      const cudaError_t e = launch_kx(GA_LOCAL, sp.tile, sp.kx, (int)sp.grid, ls);
+      fk.launch_end();
+      if (e != cudaSuccess) return GA_ERR_CUDA;
+    }
     for (int i = 0; i < nlaunch; ++i) {
       const int b = order[i];
       kps[b].bnd = bnd;
@@ -1692,7 +1846,7 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
     pending = (from_list && pending <= rerun_cap) ? 0 : 1;  // an overflowed list: rescan
     from_list = false;
   }
-  c.pairs16 += (int64_t)flat.size() * ntv - nre;
+  c.pairs16 += (int64_t)flat.size() * ntv_all - nre;
   rc = finish(c, stats, e0, e1, nq * nt);
   if (!rc && stats) {
     stats->cells = cells;

@@ -321,6 +321,31 @@ __global__ void kp_target_keys_kernel(const int64_t *t_off, int64_t nt, const ui
   if ((threadIdx.x & 31) == 0 && L > 0) atomicMax(max_len, L);
 }
 
+// Id and length of the first sorted targets, and the residues of all.
+constexpr int kKpTop = 1024;
+struct KPTop {
+  int64_t residues;
+  int2 target[kKpTop];  // (id, length); length -1 past the last valid target
+};
+__global__ void kp_top_kernel(const int64_t *t_off, int64_t nt, const int32_t *sorted, const int32_t *range, KPTop *top) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= kKpTop) return;
+  if (i == 0) top->residues = t_off[nt] - t_off[0];
+  const int id = i < range[1] - range[0] ? sorted[range[0] + i] : -1;
+  top->target[i] = make_int2(id, id >= 0 ? (int)(t_off[id + 1] - t_off[id]) : -1);
+}
+
+// Pairs of the valid queries with the first sorted targets; *range = [0, n).
+__global__ void kp_split_pairs_kernel(const int32_t *queries, int32_t nq, const int32_t *sorted, int64_t nt, int32_t n,
+                                      int32_t *list, int32_t *range) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    range[0] = 0;
+    range[1] = n;
+  }
+  if (i < n) list[i] = (int32_t)(queries[i % nq] * nt + sorted[i / nq]);
+}
+
 // Scores of pairs with an invalid query or target.
 __global__ void kp_invalid_kernel(const uint8_t *qbad, int64_t nq, const uint8_t *tbad, int64_t nt,
                                   int32_t *scores, int32_t *status) {

@@ -44,3 +44,28 @@ def test_tile_stage_and_batch_edges(A, alpha, beta, lo, hi):
     for k in (1, 12, len(qs) - 1):
         one = ga.align_cross(dev[0], dev[1][k:k + 2].contiguous(), *dev[2:], mat, alpha, beta, "local")
         assert torch.equal(one.ravel(), got[k])
+
+
+@pytest.mark.parametrize("nq,long_targets", [(1, 3), (8, 40), (30, 5)])
+def test_long_targets_beside_many_short_ones(nq, long_targets):
+    # the longest targets run as strips beside the search kernel: every pair once,
+    # invalid and empty targets as before
+    rng = np.random.default_rng(nq)
+    mat = synth.blosum62()
+    qs = [rng.integers(0, 20, size=int(n)).astype(np.uint8) for n in rng.integers(1, 700, size=nq)]
+    lens = np.concatenate([rng.integers(0, 150, size=900), rng.integers(1000, 2600, size=long_targets)])
+    ts = [rng.integers(0, 20, size=int(n)).astype(np.uint8) for n in rng.permutation(lens)]
+    longest = int(np.argmax([len(t) for t in ts]))
+    ts[longest][200:200 + len(qs[0])] = qs[0]
+    qc, qo = synth.pack_csr(qs)
+    tc, to = synth.pack_csr(ts)
+    want, _ = oracle.cross(qc, qo, tc, to, mat, 11, 1, "local", nthreads=NTHREADS)
+    want = np.asarray(want).reshape(nq, len(ts)).copy()
+    for bad in (False, True):
+        if bad:
+            tc[to[longest] + 5] = 40
+            want[:, longest] = np.iinfo(np.int32).min
+        dev = [torch.from_numpy(a).cuda() for a in (qc, qo, tc, to)]
+        got, st = ga.align_cross(*dev, mat, 11, 1, "local", stats=True)
+        assert np.array_equal(got.cpu().numpy(), want)
+        assert st["pairs_int16"] == nq * (len(ts) - bad) and (st["status"] != 0) == bad
