@@ -77,7 +77,9 @@ extern "C" {
  * fill of every pair at the cost of more registers per lane, more lanes do
  * the opposite.  concurrent = 1 runs the bins as parallel branches (side
  * streams, graph branches), so that one bin's last tasks overlap the next
- * bin's first; 0 runs them one after another on the caller's stream.
+ * bin's first; 0 runs them one after another on the caller's stream.  The
+ * tuning of a new plan (every tile, concurrent and lanes_alt 0) leaves this
+ * to the plan: parallel branches, or one launch for small capacities.
  * Every tuning gives the same (exact) scores; only the time differs. */
 typedef struct {
     uint32_t tiles16;
@@ -112,7 +114,8 @@ int ga_plan_stats(ga_plan *plan, void *stream, ga_stats *stats);
  * and keeps a candidate only when it saves more than 1 %: first dropping
  * every tile that no pair of the sample uses (one launch each; the widest
  * int16x2 tile stays, and the int32 tiles go when the sample has no int32
- * pair), then bins one after another vs concurrent, then, greedily,
+ * pair; a new plan's bins stay concurrent), then bins one after another vs
+ * concurrent, then, greedily,
  * removing one active non-empty tile at a time.  Later batches with pairs
  * in a dropped tile's range run on the next wider active tile (or the
  * intra-sequence kernel), so their scores stay exact.

@@ -881,11 +881,11 @@ struct Events {
 // takes.  Its strips pad a pair to 256, 512 or 768 columns, so it is the slower
 // kernel once the chip is full.  GB300, us a call, planned / one launch: 1,000
 // pairs of 150 residues 183 / 70, 4,000 of 100..300 349 / 164, 8,000 of 250..500
-// 480 / 444, 16,000 of 250..500 657 / 787.  A plan's default tuning runs its bins
-// in line, which loses to one launch for longer: 1,000 of 100..300 553 / 58,
-// 16,000 of 250..500 1,321 / 731, 32,000 of 150 370 / 339.
+// 480 / 444, 16,000 of 250..500 682 / 796.  In a plan's graph, where neither waits
+// for the host: 9,000 of 100..300 430 / 217, 16,000 444 / 340, 24,000 466 / 482;
+// 16,000 of 150 186 / 182, 24,000 231 / 260; 16,000 of 250..500 661 / 736.
 constexpr int64_t kKrPairs = 8192;
-constexpr int64_t kKrPlanPairs = 32768;
+constexpr int64_t kKrPlanPairs = 16384;
 
 bool kr_scoring(const Scoring &sc) { return sc.A <= 4 && std::max(sc.smax, 0) + sc.alpha <= kKxMaxStep; }
 
@@ -2080,8 +2080,12 @@ int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, cons
   ka.rerun_count = &P.small->rerun_range[1];
 
   // every bin (widest first) plus the long class, one persistent launch
-  // each; concurrent: round-robin over the side streams, joined on s
-  const bool conc = P.tune.concurrent != 0;
+  // each; concurrent: round-robin over the side streams, joined on s.  An untuned
+  // plan launches every tile, most of them for a few pairs or none, so its bins
+  // run as parallel branches.  GB300, us a replay, in line / parallel: 50,000 pairs
+  // of 100..300 1,586 / 543, 50,000 of 150 487 / 377, 20,000 of 300..900 3,942 /
+  // 3,282, 1,000 of 400..1,000 670 / 473.
+  const bool conc = P.tune.concurrent != 0 || default_tuning(P.tune);
   int nlaunch = 0, counter = 0;
   auto stream_for = [&](int i) { return conc ? P.side[i % kPlanSide] : s; };
   if (conc) {
@@ -2275,6 +2279,7 @@ int plan_autotune(PlanImpl &P, const uint8_t *qc, const int64_t *qo, const uint8
     if ((rc = live_mask(0, &l16)) || (rc = live_mask(1, &l32))) return rc;
     if (l16 != best.tiles16 || l32 != best.tiles32) {
       ga_tuning cand = best;
+      if (default_tuning(best)) cand.concurrent = 1;  // as the untuned plan runs
       // keep the widest tile of each class so that the pairs of its range
       // stay on the inter-sequence kernels
       cand.tiles16 = l16 | (best.tiles16 & (1u << (kKaNumBins - 1)));
