@@ -73,9 +73,9 @@ struct TrainParams {
 // possible step is then 32 + 64 + 64 + 64 dependent multiply-adds of a sample,
 // 256 of a parameter, and two exchanges.  Two launches per step with a thread
 // per sample and a thread per parameter took 265 us per step at a batch of 256
-// (2 blocks, then 50 blocks of uncoalesced column reads); this takes 14 us, of
-// which about 3.5 us are the forward and backward pass, 2 us the gradients
-// (both at one shared-memory wavefront per cycle), and 7 us the exchanges.
+// (2 blocks, then 50 blocks of uncoalesced column reads); this takes 10.6 us, of
+// which 2.6 us are the forward and backward pass, 2.3 us the gradients (both at one
+// shared-memory wavefront per cycle), 1.1 us Adam, and 3 us the exchanges.
 //
 // Split.  Chunks of 256 samples.  Forward and backward: each block owns SP =
 // 256 / NC samples, a warp four of them: lane l computes units l and l + 32 of
@@ -83,16 +83,18 @@ struct TrainParams {
 // serves four samples.  Gradients: block (p, q) of a 4 x NC/4 grid owns the
 // parameters of 16 units o = 16p.. and 1/(NC/4) of the inputs i of W1 and W2, a
 // 2 x 2 tile per thread, with the master value and both moments in registers
-// for the whole run.  Activations go to the blocks that own the parameters
-// they enter through distributed shared memory, a row of units per store, and
-// new weights the same way to every block.  Two cluster barriers per chunk
-// order the exchanges (activations before the gradients, and everything read
-// before it is overwritten).  The next chunk's inputs are loaded a chunk ahead.
-// The last warp takes the biases, the head and the loss.
-constexpr int kTrChunk = 256;              // samples per chunk
-constexpr int kTrS1 = kMlpIn + 4, kTrS2 = kMlpH + 4;  // padded rows of W1 and W2 in shared memory
-constexpr int kTrW1 = 0, kTrB1 = kTrW1 + kMlpH * kTrS1, kTrW2 = kTrB1 + kMlpH, kTrB2 = kTrW2 + kMlpH * kTrS2,
-              kTrW3 = kTrB2 + kMlpH, kTrB3 = kTrW3 + kMlpH, kTrWeights = kTrB3 + 4;
+// for the whole run.  The exchanges are bulk copies between the blocks' shared
+// memories, counted by an mbarrier of the receiver: a block's samples of one group
+// of units are one piece for each block that owns parameters of those units, and a
+// block's new weights are one tile for every other block.  (Stored value by value
+// into the receivers, 53 KB a step and block in pieces of 64 bytes, between cluster
+// barriers, the exchanges took 7 us: 13.8 us a step.)  The two waits order
+// everything: a block sends activations only after it has every block's weights,
+// and weights only after it has every block's activations, so what is overwritten
+// has been read; chunks without new weights end in a cluster barrier instead.  The
+// next chunk's inputs are loaded a chunk ahead.  The last warp takes the biases,
+// the head and the loss.
+constexpr int kTrChunk = 256;  // samples per chunk
 
 template <int NC>
 struct TrainShape {
@@ -103,23 +105,41 @@ struct TrainShape {
   static constexpr int N2 = 8 * (I2 / 2), N1 = 8 * (I1 / 2);  // threads with a tile of W2, of W1
   static constexpr int PER = kTrChunk / T;          // staged samples per thread
   static_assert(N2 + N1 + 32 <= T && PER * I1 == 16, "roles");
+  // Weights: W1 and W2 as the tiles of the blocks that own them (16 units x I1 or
+  // I2 inputs, padded rows), so that a block's new weights are one piece.  Row and
+  // tile strides keep row reads by 8 lanes and column reads by 32 conflict-free.
+  static constexpr int RS1 = I1 + 4, RS2 = I2 + 4, TS1 = 16 * RS1, TS2 = 16 * RS2 + (I2 == 16 ? 16 : 0);
+  static constexpr int oW1 = 0, oW2 = oW1 + NC * TS1, oB1 = oW2 + NC * TS2, oB2 = oB1 + kMlpH, oW3 = oB2 + kMlpH,
+                       oB3 = oW3 + kMlpH, kWeights = oB3 + 4;
   static constexpr int kAct = 4 * (kMlpIn + 3 * kMlpH);  // floats per warp: x, h1, h2, d2 of 4 samples
-  static constexpr int oD2 = kTrWeights + (T / 32) * kAct, oD1 = oD2 + 16 * kTrChunk,
+  // what the block sends: per group of units, its samples' rows
+  static constexpr int GS = SP * 16 + 16, GS1 = SP * I2 + (I2 == 16 ? 16 : 0);
+  static constexpr int oS2 = kWeights + (T / 32) * kAct, oS1 = oS2 + 4 * GS, oSH = oS1 + 4 * GS, oSA = oSH + 4 * GS,
+                       oSY = oSA + Q * GS1, oSR = oSY + SP;
+  // what it receives, a row per sample of the chunk
+  static constexpr int oD2 = oSR + SP, oD1 = oD2 + 16 * kTrChunk,
                        oH2 = oD1 + 16 * kTrChunk, oH1 = oH2 + 16 * kTrChunk, oX = oH1 + I2 * kTrChunk,
-                       oDY = oX + I1 * kTrChunk, oR = oDY + kTrChunk, kFloats = oR + kTrChunk;
+                       oDY = oX + I1 * kTrChunk, oR = oDY + kTrChunk, oBar = oR + kTrChunk, kFloats = oBar + 4;
+  static_assert(oW2 % 4 == 0 && oB1 % 4 == 0 && kWeights % 4 == 0 && GS % 4 == 0 && GS1 % 4 == 0 && oBar % 4 == 0,
+                "16-byte pieces");
+  static constexpr __device__ __forceinline__ int w1(int o, int i) {
+    return oW1 + (o / 16 * Q + i / I1) * TS1 + o % 16 * RS1 + i % I1;
+  }
+  static constexpr __device__ __forceinline__ int w2(int o, int i) {
+    return oW2 + (o / 16 * Q + i / I2) * TS2 + o % 16 * RS2 + i % I2;
+  }
+  // Position of parameter k.
+  static __device__ __forceinline__ int slot(int k) {
+    if (k < kOffB1) return w1(k / kMlpIn, k % kMlpIn);
+    if (k < kOffW2) return oB1 + (k - kOffB1);
+    if (k < kOffB2) return w2((k - kOffW2) / kMlpH, (k - kOffW2) % kMlpH);
+    if (k < kOffW3) return oB2 + (k - kOffB2);
+    if (k < kOffB3) return oW3 + (k - kOffW3);
+    return oB3;
+  }
   static constexpr size_t kSmem = sizeof(float) * kFloats;
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
-
-// Position of parameter k in the padded shared-memory copy.
-__device__ __forceinline__ int tr_slot(int k) {
-  if (k < kOffB1) return kTrW1 + (k / kMlpIn) * kTrS1 + k % kMlpIn;
-  if (k < kOffW2) return kTrB1 + (k - kOffB1);
-  if (k < kOffB2) return kTrW2 + ((k - kOffW2) / kMlpH) * kTrS2 + (k - kOffW2) % kMlpH;
-  if (k < kOffW3) return kTrB2 + (k - kOffB2);
-  if (k < kOffB3) return kTrW3 + (k - kOffW3);
-  return kTrB3;
-}
 
 __device__ __forceinline__ float tr_bf16(float w) { return bf16_bits_to_f32(f32_to_bf16_bits(w)); }
 
@@ -134,14 +154,16 @@ __device__ __forceinline__ void tr_adam(TrState &s, float g, const AdamArgs &a, 
   s.w = s.w - a.lr * mhat / (sqrtf(vhat) + a.eps);
 }
 
-// Dot products of units l and l + 32 with four samples: z[u][s] += sum_k
-// W[u][k] x[s][k] in index order.
-template <int N, int STRIDE>
-__device__ __forceinline__ void tr_layer(const float *W, const float *x, int l, float (&z)[2][4]) {
+// Dot products of two units with four samples: z[u][s] += sum_k W[u][k] x[s][k] in
+// index order; W0 and W1 point to the units' rows in the first of the tiles of I
+// inputs, TS apart.
+template <int N, int I, int TS>
+__device__ __forceinline__ void tr_layer(const float *W0, const float *W1, const float *x, float (&z)[2][4]) {
 #pragma unroll 4
   for (int k = 0; k < N; k += 4) {
-    const float4 wa = *reinterpret_cast<const float4 *>(W + l * STRIDE + k);
-    const float4 wc = *reinterpret_cast<const float4 *>(W + (l + 32) * STRIDE + k);
+    const int at = k / I * TS + k % I;
+    const float4 wa = *reinterpret_cast<const float4 *>(W0 + at);
+    const float4 wc = *reinterpret_cast<const float4 *>(W1 + at);
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       const float4 v = *reinterpret_cast<const float4 *>(x + s * N + k);
@@ -150,6 +172,41 @@ __device__ __forceinline__ void tr_layer(const float *W, const float *x, int l, 
     }
   }
 }
+
+// Pieces between the blocks' shared memories: one bulk copy each, counted in bytes
+// by an mbarrier of the receiver.
+__device__ __forceinline__ uint32_t tr_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t tr_peer(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void tr_copy(int rank, const float *dst, const float *src, int floats, const uint64_t *bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(tr_peer(tr_addr(dst), rank)), "r"(tr_addr(src)), "r"(4 * floats), "r"(tr_peer(tr_addr(bar), rank))
+               : "memory");
+}
+__device__ __forceinline__ void tr_bar_init(uint64_t *bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(tr_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void tr_expect(uint64_t *bar, int bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tr_addr(bar)), "r"(bytes) : "memory");
+}
+// False: the limit ran out (2 s; nothing of the kernel waits that long).
+__device__ __forceinline__ bool tr_wait(uint64_t *bar, uint32_t parity) {
+  uint32_t ok = 0;
+  const long long start = clock64();
+  while (!ok && clock64() - start < (1ll << 32))
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(tr_addr(bar)), "r"(parity)
+        : "memory");
+  return ok != 0;
+}
+// Shared memory written by this thread may be the source of a bulk copy.
+__device__ __forceinline__ void tr_publish() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 template <int NC>
 __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __grid_constant__ TrainParams p) {
@@ -160,12 +217,13 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
   const int rank = (int)cluster.block_rank(), tid = threadIdx.x, l = tid & 31, warp = tid >> 5;
   const int bp = rank / S::Q, bq = rank % S::Q;
   float *W = tr_smem;
-  float *xs = tr_smem + kTrWeights + warp * S::kAct, *h1s = xs + 4 * kMlpIn, *h2s = h1s + 4 * kMlpH,
+  uint64_t *bar_a = reinterpret_cast<uint64_t *>(tr_smem + S::oBar), *bar_w = bar_a + 1;
+  float *xs = tr_smem + S::kWeights + warp * S::kAct, *h1s = xs + 4 * kMlpIn, *h2s = h1s + 4 * kMlpH,
         *d2s = h2s + 4 * kMlpH;
   const bool upd = p.a.update != 0;
 
   for (int k = tid; k < kMlpParams; k += S::T)
-    W[tr_slot(k)] = upd ? tr_bf16(p.master[k]) : bf16_bits_to_f32(p.wb_in[k]);
+    W[S::slot(k)] = upd ? tr_bf16(p.master[k]) : bf16_bits_to_f32(p.wb_in[k]);
 
   // ---- the parameters of this thread --------------------------------------
   // role 0: 2 x 2 tile of W2, 1: of W1, 2: one parameter or the loss, 3: none
@@ -226,16 +284,16 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
   int bad_idx = 0;
   // the index is only loaded here; it is checked where the inputs are read, so
   // that nothing waits for it (kNone: no sample at this place)
-  constexpr int64_t kNone = INT64_MIN;
-  auto sample_of = [&](int step, int c0, int b) -> int64_t {
+  constexpr int32_t kNone = INT32_MIN;
+  auto sample_of = [&](int step, int c0, int b) -> int32_t {
     if (step >= p.steps || b >= ::min(kTrChunk, p.B - c0)) return kNone;
-    return p.idx ? (int64_t)p.idx[(int64_t)step * p.B + c0 + b] : (int64_t)(c0 + b);
+    return p.idx ? p.idx[(int64_t)step * p.B + c0 + b] : c0 + b;
   };
   auto own_base = [&](int cb) -> int {  // first sample of this warp in a chunk of cb, or >= cb
     const int spc = ((cb + NC - 1) / NC + 3) & ~3;
     return 4 * warp < spc ? rank * spc + 4 * warp : kTrChunk;
   };
-  int64_t own_s[4], con_s[S::PER];
+  int32_t own_s[4], con_s[S::PER];
   auto read_idx = [&](int step, int c0) {
     const int sb = own_base(::min(kTrChunk, p.B - c0));
 #pragma unroll
@@ -248,7 +306,7 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
       const bool in = own_s[s] >= 0 && own_s[s] < p.nsamples;
-      xv[s] = in ? p.x[own_s[s] * kMlpIn + l] : 0.f;
+      xv[s] = in ? p.x[(int64_t)own_s[s] * kMlpIn + l] : 0.f;
       ok |= (in ? 1u : 0u) << s;
       if ((l & 3) == s) tv = in ? p.target[own_s[s]] : 0.f;
     }
@@ -257,24 +315,41 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
       const bool in = con_s[j] >= 0 && con_s[j] < p.nsamples;
       bad_idx |= !in && con_s[j] != kNone;
 #pragma unroll
-      for (int i = 0; i < S::I1; ++i) xc[j][i] = in ? p.x[con_s[j] * kMlpIn + S::I1 * bq + i] : 0.f;
+      for (int i = 0; i < S::I1; ++i) xc[j][i] = in ? p.x[(int64_t)con_s[j] * kMlpIn + S::I1 * bq + i] : 0.f;
     }
   };
   read_idx(0, 0);
   read_x();
-  cluster.sync();  // every block of the cluster runs, its weights are in place
+  if (tid == 0) {
+    tr_bar_init(bar_a);
+    tr_bar_init(bar_w);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  cluster.sync();  // every block of the cluster runs, its weights and barriers are in place
+  uint32_t parity_a = 0, parity_w = 0;
+  bool alive = true;  // no wait has run out
+  // bytes of the weights that the other blocks send
+  constexpr int kOwnTiles = 16 * (S::RS1 + S::RS2);
+  const int w_bytes = 4 * ((NC - 1) * kOwnTiles + (bq == 0 ? 3 : 4) * 32 + (bq == 1 ? 3 : 4) * 16 + (rank == 1 ? 0 : 4));
 
   for (int step = 0; step < p.steps; ++step) {
+    if (upd && tid == 0) tr_expect(bar_w, w_bytes);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
     const float2 coef = upd ? p.coef[step] : make_float2(0.f, 0.f);
     for (int c0 = 0; c0 < p.B; c0 += kTrChunk) {
       const int cb = ::min(kTrChunk, p.B - c0);
       const int sb = own_base(cb);
+      if (tid == 0) {
+        const int rows = (cb + 3) & ~3;
+        tr_expect(bar_a, 4 * rows * (S::I2 + 32 + (bq == 0 ? 17 : 0) + (rank == 1 ? 2 : 0)));
+      }
       // ---- forward and backward of this warp's four samples -----------------
 #pragma unroll
       for (int j = 0; j < S::PER; ++j)
 #pragma unroll
-        for (int i = 0; i < S::I1; ++i) tr_smem[S::oX + (tid + j * S::T) * S::I1 + i] = xc[j][i];
+        for (int i = 0; i < S::I1; i += 4)
+          *reinterpret_cast<float4 *>(tr_smem + S::oX + (tid + j * S::T) * S::I1 + i) =
+              make_float4(xc[j][i], xc[j][i + 1], xc[j][i + 2], xc[j][i + 3]);
 #pragma unroll
       for (int s = 0; s < 4; ++s) xs[s * kMlpIn + l] = xv[s];
       const float target = tv;
@@ -286,10 +361,10 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
         float z[2][4], h1[2][4], h2[2][4], d2[2][4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          z[0][s] = W[kTrB1 + l];
-          z[1][s] = W[kTrB1 + l + 32];
+          z[0][s] = W[S::oB1 + l];
+          z[1][s] = W[S::oB1 + l + 32];
         }
-        tr_layer<kMlpIn, kTrS1>(W + kTrW1, xs, l, z);
+        tr_layer<kMlpIn, S::I1, S::TS1>(W + S::w1(l, 0), W + S::w1(l + 32, 0), xs, z);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -297,20 +372,20 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
         __syncwarp();
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          z[0][s] = W[kTrB2 + l];
-          z[1][s] = W[kTrB2 + l + 32];
+          z[0][s] = W[S::oB2 + l];
+          z[1][s] = W[S::oB2 + l + 32];
         }
-        tr_layer<kMlpH, kTrS2>(W + kTrW2, h1s, l, z);
+        tr_layer<kMlpH, S::I2, S::TS2>(W + S::w2(l, 0), W + S::w2(l + 32, 0), h1s, z);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
           for (int s = 0; s < 4; ++s) h2s[s * kMlpH + l + 32 * u] = h2[u][s] = fmaxf(z[u][s], 0.f);
         __syncwarp();
-        float y = W[kTrB3];
+        float y = W[S::oB3];
         const float *hv = h2s + (l & 3) * kMlpH;
 #pragma unroll 4
         for (int o = 0; o < kMlpH; o += 4) {
-          const float4 w = *reinterpret_cast<const float4 *>(W + kTrW3 + o);
+          const float4 w = *reinterpret_cast<const float4 *>(W + S::oW3 + o);
           const float4 v = *reinterpret_cast<const float4 *>(hv + o);
           y = fmaf(w.w, v.w, fmaf(w.z, v.z, fmaf(w.y, v.y, fmaf(w.x, v.x, y))));
         }
@@ -323,7 +398,7 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
         for (int u = 0; u < 2; ++u)
 #pragma unroll
           for (int s = 0; s < 4; ++s)
-            d2s[s * kMlpH + l + 32 * u] = d2[u][s] = h2[u][s] > 0.f ? dys[s] * W[kTrW3 + l + 32 * u] : 0.f;
+            d2s[s * kMlpH + l + 32 * u] = d2[u][s] = h2[u][s] > 0.f ? dys[s] * W[S::oW3 + l + 32 * u] : 0.f;
         __syncwarp();
 #pragma unroll
         for (int s = 0; s < 4; ++s) z[0][s] = z[1][s] = 0.f;
@@ -332,8 +407,8 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
           float wa[4], wc[4];
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            wa[j] = W[kTrW2 + (o + j) * kTrS2 + l];
-            wc[j] = W[kTrW2 + (o + j) * kTrS2 + l + 32];
+            wa[j] = W[S::w2(o + j, l)];
+            wc[j] = W[S::w2(o + j, l + 32)];
           }
 #pragma unroll
           for (int s = 0; s < 4; ++s) {
@@ -342,36 +417,52 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
             z[1][s] = fmaf(d.w, wc[3], fmaf(d.z, wc[2], fmaf(d.y, wc[1], fmaf(d.x, wc[0], z[1][s]))));
           }
         }
-        // ---- to the blocks that own the parameters ---------------------------
-        auto put = [&](int dst, int at, float v) { *cluster.map_shared_rank(tr_smem + at, dst) = v; };
+        // ---- staged for the blocks that own the parameters -------------------
+        const int row = 4 * warp;
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
-          const int b = sb + s;
           const bool keep = (valid >> s) & 1u;  // an invalid sample adds nothing
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const int unit = l + 32 * u, ub = unit / 16 * S::Q, uo = b * 16 + unit % 16;
-            const float e1 = keep ? h1[u][s] : 0.f, e2 = keep ? d2[u][s] : 0.f;
-            const float e3 = keep && h1[u][s] > 0.f ? z[u][s] : 0.f;
-#pragma unroll
-            for (int r4 = 0; r4 < 4; ++r4)
-              put(r4 * S::Q + unit / S::I2, S::oH1 + b * S::I2 + unit % S::I2, e1);
-#pragma unroll
-            for (int q = 0; q < S::Q; ++q) {
-              put(ub + q, S::oD2 + uo, e2);
-              put(ub + q, S::oD1 + uo, e3);
-            }
-            put(ub, S::oH2 + uo, keep ? h2[u][s] : 0.f);
+            const int unit = l + 32 * u, at = unit / 16 * S::GS + (row + s) * 16 + unit % 16;
+            tr_smem[S::oS2 + at] = keep ? d2[u][s] : 0.f;
+            tr_smem[S::oS1 + at] = keep && h1[u][s] > 0.f ? z[u][s] : 0.f;
+            tr_smem[S::oSH + at] = keep ? h2[u][s] : 0.f;
+            tr_smem[S::oSA + unit / S::I2 * S::GS1 + (row + s) * S::I2 + unit % S::I2] = keep ? h1[u][s] : 0.f;
           }
         }
-        if (l < 20) {  // the head's error signal to the blocks that own the head, the error to the loss
-          const int s = l & 3, d = l >> 2;
-          put(d < 4 ? d * S::Q : 1, S::oDY + sb + s, dy);
-          if (d == 4) put(1, S::oR + sb + s, r);
+        if (l < 4) {  // the head's error signal, the error
+          tr_smem[S::oSY + row + l] = dy;
+          tr_smem[S::oSR + row + l] = r;
+        }
+        tr_publish();
+      }
+      __syncthreads();
+      {
+        // this block's rows: b0 .. b0 + n of the chunk
+        const int spc = ((cb + NC - 1) / NC + 3) & ~3, b0 = rank * spc;
+        const int n = ::min(spc, ::max(0, (cb - b0 + 3) & ~3));
+        if (n > 0) {
+          // a kind of piece per warp, a block per lane
+          const int d = l, kind = warp, dp = d / S::Q, dq = d % S::Q;
+          if (d < NC && kind < 4) {
+            if (kind == 0) tr_copy(d, tr_smem + S::oD2 + b0 * 16, tr_smem + S::oS2 + dp * S::GS, 16 * n, bar_a);
+            else if (kind == 1) tr_copy(d, tr_smem + S::oD1 + b0 * 16, tr_smem + S::oS1 + dp * S::GS, 16 * n, bar_a);
+            else if (kind == 2)
+              tr_copy(d, tr_smem + S::oH1 + b0 * S::I2, tr_smem + S::oSA + dq * S::GS1, S::I2 * n, bar_a);
+            else if (dq == 0) {
+              tr_copy(d, tr_smem + S::oH2 + b0 * 16, tr_smem + S::oSH + dp * S::GS, 16 * n, bar_a);
+              tr_copy(d, tr_smem + S::oDY + b0, tr_smem + S::oSY, n, bar_a);
+            } else if (d == 1) {
+              tr_copy(d, tr_smem + S::oDY + b0, tr_smem + S::oSY, n, bar_a);
+              tr_copy(d, tr_smem + S::oR + b0, tr_smem + S::oSR, n, bar_a);
+            }
+          }
         }
       }
       read_x();  // the next chunk's inputs arrive while the gradients run
-      cluster.sync();
+      if (alive) alive = tr_wait(bar_a, parity_a);
+      parity_a ^= 1;
       // ---- gradients, in sample order ---------------------------------------
       if (role < 2) {
         // eight samples are loaded while the eight before them are summed
@@ -425,23 +516,39 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
             tr_adam(st[e], acc[e], p.a, coef);
             n[e] = tr_bf16(st[e].w);
           }
-          const int at0 = tr_slot(par[0]), at1 = tr_slot(par[2]);
-#pragma unroll
-          for (int r = 0; r < NC; ++r) {
-            *reinterpret_cast<float2 *>(cluster.map_shared_rank(W + at0, r)) = make_float2(n[0], n[1]);
-            *reinterpret_cast<float2 *>(cluster.map_shared_rank(W + at1, r)) = make_float2(n[2], n[3]);
-          }
+          *reinterpret_cast<float2 *>(W + S::slot(par[0])) = make_float2(n[0], n[1]);
+          *reinterpret_cast<float2 *>(W + S::slot(par[2])) = make_float2(n[2], n[3]);
         } else if (upd && role == 2 && !is_loss) {
           tr_adam(st[0], acc[0], p.a, coef);
-          const float n = tr_bf16(st[0].w);
-          const int at = tr_slot(par[0]);
-#pragma unroll
-          for (int r = 0; r < NC; ++r) *cluster.map_shared_rank(W + at, r) = n;
+          W[S::slot(par[0])] = tr_bf16(st[0].w);
         }
       }
-      cluster.sync();
+      if (last && upd) {
+        // the new weights to every other block; what it received has been read
+        tr_publish();
+        __syncthreads();
+        const int d = l, kind = warp;
+        if (d < NC && d != rank) {
+          const float *w2 = W + S::oW2 + rank * S::TS2, *w1 = W + S::oW1 + rank * S::TS1;
+          if (kind == 0) tr_copy(d, w2, w2, 16 * S::RS2, bar_w);
+          else if (kind == 1) tr_copy(d, w1, w1, 16 * S::RS1, bar_w);
+          else if (kind == 2 && bq < 2) {
+            const float *v = W + (bq == 0 ? S::oB2 : S::oB1) + 16 * bp;
+            tr_copy(d, v, v, 16, bar_w);
+          } else if (kind == 3 && (bq == 0 || rank == 1)) {
+            const float *v = W + (bq == 0 ? S::oW3 + 16 * bp : S::oB3);
+            tr_copy(d, v, v, bq == 0 ? 16 : 4, bar_w);
+          }
+        }
+        if (alive) alive = tr_wait(bar_w, parity_w);
+        parity_w ^= 1;
+      } else if (!last) {
+        cluster.sync();  // everything read before it is overwritten
+      }
     }
   }
+  cluster.sync();  // no block leaves while another copies from or to it
+  if (!alive && p.status) set_status(p.status, GA_ERR_CUDA);
   if (bad_idx && p.status) set_status(p.status, GA_ERR_ARG);
   if (upd)
     for (int e = 0; e < 4; ++e)
@@ -515,14 +622,13 @@ cudaError_t launch_train(const TrainParams &p, cudaStream_t s, bool only_if_it_f
   return cudaLaunchKernelEx(&cfg, mlp_train_kernel<NC>, p);
 }
 
-// Cluster size: 8 blocks below 96 samples a step, where a chunk keeps few warps
-// busy and a smaller cluster exchanges faster (GB300, us per step, 16 / 8
-// blocks: 8.5 / 7.8 at 16 samples, 8.9 / 8.8 at 64, 10.2 / 10.8 at 128, 13.8 /
-// 16.2 at 256, 46 / 58 at 1024); 8 is also the portable size where a device
+// Cluster size: 8 blocks below 32 samples a step, where a chunk keeps few warps
+// busy (GB300, us per step, 16 / 8 blocks: 6.9 / 6.7 at 16 samples, 7.1 / 7.3 at
+// 32, 7.7 / 8.1 at 64, 7.8 / 9.1 at 95); 8 is also the portable size where a device
 // places no cluster of 16.  The results are the same.
 cudaError_t enqueue_train(const TrainParams &p, cudaStream_t s) {
   bool launched = false;
-  if (p.B >= 96) {
+  if (p.B >= 32) {
     const cudaError_t e = launch_train<16>(p, s, true, &launched);
     if (e != cudaSuccess || launched) return e;
   }
