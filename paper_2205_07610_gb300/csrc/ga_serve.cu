@@ -284,6 +284,14 @@ struct ga_server {
 namespace ga {
 namespace {
 
+// Requests of a tick with a sequence of this length are queued before the others: a
+// burst otherwise ends with the chain of rows of a long request that came late.
+// GB300, bursts of lengths up to 50,000, ms to the last result in arrival order /
+// from 32,768 on first / from 8,192 on first: 4,000 requests 19.5 / 16.5 / 16.7, 2,000
+// 12.1 / 11.8 / 12.0, 300 and fewer the same; half of the 4,000 are done after 6.0 /
+// 6.7 / 9.3, so the shorter ones keep their place.
+constexpr int64_t kSvLongFirst = 32768;
+
 // One scheduler tick: admit, publish, relaunch, collect.  Returns whether
 // anything happened.
 bool sched_tick(ga_server *S) {
@@ -386,11 +394,13 @@ bool sched_tick(ga_server *S) {
       r.scoring = a.pd.scoring;
       r.nstrips = f.nstrips;
       r.score = a.pd.mode == kModeGlobal ? INT_MIN : 0;
-      S->stage_tasks[k] = make_int2(a.slot, 0);
-      k += 1;
       off += f.seq_bytes;
     }
     flush_run();
+    // queue order: the tick's long requests first
+    for (const bool is_long : {true, false})
+      for (const Adm &a : admit)
+        if ((std::max(a.m, a.n) >= kSvLongFirst) == is_long) S->stage_tasks[k++] = make_int2(a.slot, 0);
     t_a = S->now_ns();
     const int64_t first_slot = admit[0].slot;
     const int64_t n1 = std::min<int64_t>((int64_t)admit.size(), S->req_cap - first_slot);
