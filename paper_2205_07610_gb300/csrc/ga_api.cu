@@ -526,6 +526,13 @@ int plan_bin_count(const ChunkPlan &p, int cls, int bin) {
   return p.r.ranges[2 * key + 1] - p.r.ranges[2 * key];
 }
 
+// Zeroed words before the edges of a strip launch over n pairs: the pairs' states,
+// the task counter and count, the scratch of the task list.
+size_t kx_zeroed(int64_t n) { return sizeof(KXPairState) * (size_t)n + 16 + sizeof(KXTaskScratch); }
+KXTaskScratch *kx_scratch(char *zero, int64_t n) {
+  return reinterpret_cast<KXTaskScratch *>(zero + sizeof(KXPairState) * (size_t)n + 16);
+}
+
 // Strip launch of a plan's long class: the task list and the zeroed edge words,
 // one buffer of (shorter sequence + 1) words per pair.  Left to the kernels that
 // run a pair on one warp where the relative int16 cells of the scoring are not
@@ -540,7 +547,7 @@ int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   const int64_t W = 64 * kKxTileK[tile], ntasks = strips[kKxTileK[tile] / 4 - 1];
   if (p.r.rmax_long > W * kKxMaxStrips || ntasks > (1 << 30) || ls.rows > (4ull << 30) / 8) return GA_OK;
   const int64_t cnt = p.long_cnt;
-  const size_t head = sizeof(KXPairState) * (size_t)cnt + 16, bytes = head + 8 * (size_t)ls.rows;
+  const size_t head = kx_zeroed(cnt), bytes = head + 8 * (size_t)ls.rows;
   char *zero = c.al.try_get<char>(bytes);
   int2 *tasks = zero ? c.al.try_get<int2>((size_t)ntasks) : nullptr;
   int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)cnt) : nullptr;
@@ -582,9 +589,10 @@ int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   kt.tasks = tasks;
   kt.edge_off = edge_off;
   if (cudaMemsetAsync(zero, 0, bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
-  kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
-  ++c.launches;
-  if (cudaGetLastError() != cudaSuccess) return GA_ERR_CUDA;
+  kt.scratch = kx_scratch(zero, cnt);
+  kt.state = k.state;
+  if (launch_kx_tasks(kt, cnt, c.s) != cudaSuccess) return GA_ERR_CUDA;
+  c.launches += 2;
   p.kx_tile = tile;
   return GA_OK;
 }
@@ -1256,7 +1264,7 @@ struct BandRun {
     const int64_t W = 64 * kKxTileK[f.tile];
     if (longest > W * kKxMaxStrips || sums.rows > (4ull << 30) / 8) return GA_OK;
     f.cap = strips[kKxTileK[f.tile] / 4 - 1];
-    f.bytes = sizeof(KXPairState) * (size_t)npairs + 16 + 8 * (size_t)sums.rows;
+    f.bytes = kx_zeroed(npairs) + 8 * (size_t)sums.rows;
     f.zero = c.al.try_get<char>(f.bytes);
     if (f.zero) f.tasks = c.al.try_get<int2>((size_t)f.cap);
     if (f.tasks) f.edge_off = c.al.try_get<int64_t>((size_t)npairs);
@@ -1312,7 +1320,7 @@ struct BandRun {
     k.counter = reinterpret_cast<int32_t *>(f.zero + sizeof(KXPairState) * (size_t)npairs);
     k.ntasks_dev = k.counter + 1;
     k.edge_off = f.edge_off;
-    k.edges = reinterpret_cast<unsigned long long *>(f.zero + sizeof(KXPairState) * (size_t)npairs + 16);
+    k.edges = reinterpret_cast<unsigned long long *>(f.zero + kx_zeroed(npairs));
     k.scores = kc.scores;
     k.status = &c.small->status;
     std::memcpy(k.tables, c.sc.tables, sizeof(k.tables));
@@ -1330,7 +1338,9 @@ struct BandRun {
     kt.edge_off = f.edge_off;
     kt.ntasks = k.counter + 1;
     if (cudaMemsetAsync(f.zero, 0, f.bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
-    kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
+    kt.scratch = kx_scratch(f.zero, npairs);
+    kt.state = k.state;
+    if (launch_kx_tasks(kt, npairs, c.s) != cudaSuccess) return GA_ERR_CUDA;
     int occ = 0;
     if (launch_kx(GA_GLOBAL, f.tile, k, 0, c.s, &occ) != cudaSuccess) return GA_ERR_CUDA;
     const int kgrid = (int)std::min<int64_t>((f.cap + kKxWarps - 1) / kKxWarps, (int64_t)c.nsm * std::max(occ, 1));
@@ -1367,7 +1377,7 @@ struct BandRun {
     c.dp_begin();
     e = launch_kz(kc, grid, c.s);
     c.dp_end();
-    c.launches += 2;
+    c.launches += 3;
     return e == cudaSuccess ? GA_OK : GA_ERR_CUDA;
   }
 
@@ -1513,7 +1523,7 @@ struct KpSplit {
 };
 
 // Chooses the number of targets, in cycles: strips as estimated by kx_choose and
-// 30k and 8 a pair for their task list, then the search kernel's remaining work and
+// 15k and 1 a pair for their task list, then the search kernel's remaining work and
 // twice its longest remaining chain (its launches start one after another once the
 // chip is full), as sides of a right angle; 3 % less than no split or none.  GB300,
 // ms, search kernel alone / so split: 4 queries x 500 targets 1.53 / 0.56, 8 x 2,000
@@ -1553,7 +1563,7 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
       int tile = 0;
       if (r > 0) {
         tile = kx_choose(GA_LOCAL, true, longest, strips, c.nsm, &kx);
-        kx += 30e3 + 8.0 * r * nq;
+        kx += 15e3 + 1.0 * r * nq;
         if (longest > 64 * kKxTileK[tile] * kKxMaxStrips || rows > (1ll << 30) / 8) return;
       }
       const bool none_left = n < 0 || (r < kKpTop && n == 0);
@@ -1580,7 +1590,7 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
 // workspace the search kernel keeps them.
 int kp_split_prepare(Call &c, const SetView &Q, const SetView &T, int64_t nt, const int32_t *queries, int64_t nqv,
                      const int32_t *sorted, int32_t *scores, KpSplit &sp) {
-  const size_t head = sizeof(KXPairState) * (size_t)sp.npairs + 16, bytes = head + 8 * (size_t)sp.rows;
+  const size_t head = kx_zeroed(sp.npairs), bytes = head + 8 * (size_t)sp.rows;
   char *zero = c.al.try_get<char>(bytes);
   int2 *tasks = zero ? c.al.try_get<int2>((size_t)sp.strips) : nullptr;
   int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)sp.npairs) : nullptr;
@@ -1625,9 +1635,10 @@ int kp_split_prepare(Call &c, const SetView &Q, const SetView &T, int64_t nt, co
   kt.tasks = tasks;
   kt.edge_off = edge_off;
   if (cudaMemsetAsync(zero, 0, bytes, c.s) != cudaSuccess) return GA_ERR_CUDA;
-  kx_tasks_kernel<<<1, 1024, 0, c.s>>>(kt);
-  c.launches += 2;
-  return cudaGetLastError() == cudaSuccess ? GA_OK : GA_ERR_CUDA;
+  kt.scratch = kx_scratch(zero, sp.npairs);
+  kt.state = k.state;
+  c.launches += 3;
+  return launch_kx_tasks(kt, sp.npairs, c.s) == cudaSuccess ? GA_OK : GA_ERR_CUDA;
 }
 
 int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, int64_t nq,

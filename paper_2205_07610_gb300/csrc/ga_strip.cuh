@@ -70,7 +70,7 @@ constexpr int kKxSigRow = 9;          // words of a score vector in shared memor
 constexpr int64_t kKxWaitNs = 10ll * 1000 * 1000 * 1000;
 
 struct KXPairState {  // one per pair, zeroed before the launch
-  int32_t score, done, status, pad;
+  int32_t score, done, status, nstrips;  // nstrips: set by the task list
 };
 
 struct KXParams {
