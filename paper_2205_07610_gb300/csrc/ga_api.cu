@@ -224,6 +224,12 @@ struct Readback {
   int32_t ranges[2 * kClassesSorted * kBins];
 };
 
+__global__ void ends_kernel(const int64_t *q_off, int64_t nq, const int64_t *t_off, int64_t nt, int64_t *ends) {
+  const int k = threadIdx.x;
+  const int64_t *off = k < 2 ? q_off : t_off;
+  if (k < 4 && off) ends[k] = off[k & 1 ? (k < 2 ? nq : nt) : 0];
+}
+
 __global__ void fill_off_kernel(int64_t *off, int64_t a, int64_t b) {
   off[0] = a;
   off[1] = b;
@@ -317,16 +323,31 @@ int setup_sort(Call &c) {
   return c.al.failed ? GA_ERR_OOM : GA_OK;
 }
 
-// Validate + pack one sequence set.  Reads back the total residue count.
-// Residue range [off[0], off[nseq]) of a set, when the caller knows it on
-// the host (otherwise it is read back from the device offsets).
+// Residue range [off[0], off[nseq]) of a set, when the host knows it.
 struct KnownRange {
   bool known = false;
   int64_t start = 0, total = 0;
 };
 
+// Reads both sets' ranges back from the device offsets, in one round trip.
+int read_ranges(Call &c, const int64_t *q_off, int64_t nq, const int64_t *t_off, int64_t nt, KnownRange *qr,
+                KnownRange *tr) {
+  if ((qr->known || nq == 0) && (tr->known || nt == 0)) return GA_OK;
+  ends_kernel<<<1, 32, 0, c.s>>>(nq ? q_off : nullptr, nq, nt ? t_off : nullptr, nt, c.small->ends);
+  ++c.launches;
+  int64_t *h = (int64_t *)pinned_scratch();
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(h, c.small->ends, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
+      cudaStreamSynchronize(c.s) != cudaSuccess)
+    return GA_ERR_CUDA;
+  if (!qr->known) *qr = KnownRange{true, h[0], h[1]};
+  if (!tr->known) *tr = KnownRange{true, h[2], h[3]};
+  return GA_OK;
+}
+
+// Validate + pack one sequence set of a known range.
 int prepare_set(Call &c, const uint8_t *codes, const int64_t *off, int64_t nseq, uint32_t **packed,
-                uint8_t **bad, int32_t *invalid, KnownRange kr = KnownRange(), uint32_t **packed5 = nullptr) {
+                uint8_t **bad, int32_t *invalid, const KnownRange &kr, uint32_t **packed5 = nullptr) {
   *bad = c.al.get<uint8_t>((size_t)nseq + 1);
   *packed = nullptr;
   if (packed5) *packed5 = nullptr;
@@ -334,18 +355,8 @@ int prepare_set(Call &c, const uint8_t *codes, const int64_t *off, int64_t nseq,
   if (nseq == 0) return GA_OK;
   // the set's residues are codes[off[0] .. off[nseq]) (off[0] > 0 when the
   // set is a chunk of a larger buffer); packed words keep absolute positions
-  int64_t h0 = kr.start, h1 = kr.total;
-  if (!kr.known) {
-    int64_t *h = (int64_t *)pinned_scratch();
-    if (cudaMemcpyAsync(h, off, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
-        cudaMemcpyAsync(h + 1, off + nseq, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s) != cudaSuccess ||
-        cudaStreamSynchronize(c.s) != cudaSuccess)
-      return GA_ERR_CUDA;
-    h0 = h[0];
-    h1 = h[1];
-  }
-  const int64_t total = std::max<int64_t>(h1, 0);
-  const int64_t start = std::min(std::max<int64_t>(h0, 0), total);
+  const int64_t total = std::max<int64_t>(kr.total, 0);
+  const int64_t start = std::min(std::max<int64_t>(kr.start, 0), total);
   if (c.dna) {
     *packed = c.al.get<uint32_t>((size_t)(total / 16 + 2));
     if (c.al.failed) return GA_ERR_OOM;
@@ -379,6 +390,14 @@ struct SetView {
   uint32_t *packed;
   uint8_t *bad;
 };
+
+// Both sets of a call; t_packed5: the targets packed 5 bits each as well.
+int prepare_sets(Call &c, SetView &Q, int64_t nq, SetView &T, int64_t nt, KnownRange qr = KnownRange(),
+                 KnownRange tr = KnownRange(), uint32_t **t_packed5 = nullptr) {
+  if (int rc = read_ranges(c, Q.off, nq, T.off, nt, &qr, &tr)) return rc;
+  if (int rc = prepare_set(c, Q.codes, Q.off, nq, &Q.packed, &Q.bad, &c.small->invalid_q, qr)) return rc;
+  return prepare_set(c, T.codes, T.off, nt, &T.packed, &T.bad, &c.small->invalid_t, tr, t_packed5);
+}
 
 // The DP launches of one call on the device's side streams (two or more
 // launches), or in order on the caller's stream.
@@ -893,6 +912,10 @@ struct Events {
 // for the host: 9,000 of 100..300 430 / 217, 16,000 444 / 340, 24,000 466 / 482;
 // 16,000 of 150 186 / 182, 24,000 231 / 260; 16,000 of 250..500 661 / 736.
 constexpr int64_t kKrPairs = 8192;
+// More pairs in one mode, by the residues of both sets: 9,000 of 100..300 375 / 278,
+// 12,000 379 / 335, 16,000 of 150 253 / 245; 10,000 of 200..300 311 / 353, 9,000 of
+// 250..300 302 / 372, 25,000 of 60..120 217 / 249.
+constexpr int64_t kKrPairsMore = 16384, kKrResidues = 4800000;
 constexpr int64_t kKrPlanPairs = 16384;
 
 bool kr_scoring(const Scoring &sc) { return sc.A <= 4 && std::max(sc.smax, 0) + sc.alpha <= kKxMaxStep; }
@@ -965,7 +988,12 @@ int batch_modes_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t
   Events ev(stats != nullptr, c.s);
   if ((rc = setup(c))) return rc;
   int32_t done_len = 0;
-  if (npairs > 0 && npairs <= kKrPairs && !force_long && kr_scoring(c.sc)) {
+  bool small = npairs > 0 && npairs <= (nmodes == 1 ? kKrPairsMore : kKrPairs) && !force_long && kr_scoring(c.sc);
+  if (small && npairs > kKrPairs) {  // by its residues, which planning needs as well
+    if ((rc = read_ranges(c, q_off, npairs, t_off, npairs, &qr, &tr))) return rc;
+    small = (qr.total - qr.start) + (tr.total - tr.start) <= kKrResidues;
+  }
+  if (small) {
     int32_t left = 0;
     rc = small_batch(c, q_codes, q_off, t_codes, t_off, npairs, modes, nmodes, scores, score_stride, &left, &qr, &tr);
     if (rc) return rc;
@@ -974,8 +1002,7 @@ int batch_modes_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t
   }
   if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
-  if ((rc = prepare_set(c, q_codes, q_off, npairs, &Q.packed, &Q.bad, &c.small->invalid_q, qr))) return rc;
-  if ((rc = prepare_set(c, t_codes, t_off, npairs, &T.packed, &T.bad, &c.small->invalid_t, tr))) return rc;
+  if ((rc = prepare_sets(c, Q, npairs, T, npairs, qr, tr))) return rc;
   // one plan per mode (own sort buffers and plan state), all read back with
   // one synchronisation and launched in one fork / join
   ChunkPlan ps[8];
@@ -1123,8 +1150,7 @@ struct BandRun {
   int prepare() {
     int rc;
     if ((rc = setup_sort(c))) return rc;
-    if ((rc = prepare_set(c, Q.codes, Q.off, npairs, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
-    if ((rc = prepare_set(c, T.codes, T.off, npairs, &T.packed, &T.bad, &c.small->invalid_t))) return rc;
+    if ((rc = prepare_sets(c, Q, npairs, T, npairs))) return rc;
     keys = c.al.get<uint32_t>((size_t)npairs);
     sorted = c.al.get<int32_t>((size_t)npairs);
     return c.al.failed ? GA_ERR_OOM : GA_OK;
@@ -1407,8 +1433,7 @@ int features_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t
   if ((rc = setup(c))) return rc;
   if (npairs == 0) return finish(c, stats, ev.e0, ev.e1, 0);
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
-  if ((rc = prepare_set(c, q_codes, q_off, npairs, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
-  if ((rc = prepare_set(c, t_codes, t_off, npairs, &T.packed, &T.bad, &c.small->invalid_t))) return rc;
+  if ((rc = prepare_sets(c, Q, npairs, T, npairs))) return rc;
   BandFeatParams fp{};
   fp.packed_q = Q.packed;
   fp.packed_t = T.packed;
@@ -1647,10 +1672,8 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   int rc;
   if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
-  if ((rc = prepare_set(c, q_codes, q_off, nq, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
   uint32_t *t_packed5 = nullptr;
-  if ((rc = prepare_set(c, t_codes, t_off, nt, &T.packed, &T.bad, &c.small->invalid_t, KnownRange(), &t_packed5)))
-    return rc;
+  if ((rc = prepare_sets(c, Q, nq, T, nt, KnownRange(), KnownRange(), &t_packed5))) return rc;
   if (nt >= (1ll << 31) - 64 || nq * nt >= (1ll << 31) - 64) return GA_ERR_ARG;
   uint32_t *keys = c.al.get<uint32_t>((size_t)nt);
   int32_t *sorted = c.al.get<int32_t>((size_t)nt);
@@ -2568,8 +2591,7 @@ int ga_align_cross(const uint8_t *q_codes, const int64_t *q_off, int64_t nq, con
     return cross_protein_local(c, q_codes, q_off, nq, t_codes, t_off, nt, scores, stats, ev.e0, ev.e1);
   if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
-  if ((rc = prepare_set(c, q_codes, q_off, nq, &Q.packed, &Q.bad, &c.small->invalid_q))) return rc;
-  if ((rc = prepare_set(c, t_codes, t_off, nt, &T.packed, &T.bad, &c.small->invalid_t))) return rc;
+  if ((rc = prepare_sets(c, Q, nq, T, nt))) return rc;
   const int64_t kChunk = 1 << 22;
   const int64_t qpc = std::max<int64_t>(1, std::min<int64_t>(nq, kChunk / nt));
   const int64_t cap = qpc * nt;
