@@ -209,7 +209,7 @@ __device__ __forceinline__ bool tr_wait(uint64_t *bar, uint32_t parity) {
 __device__ __forceinline__ void tr_publish() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 template <int NC>
-__global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __grid_constant__ TrainParams p) {
+__global__ void __launch_bounds__(TrainShape<NC>::T, 1) mlp_train_kernel(const __grid_constant__ TrainParams p) {
   using S = TrainShape<NC>;
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) float tr_smem[];
@@ -326,8 +326,8 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   cluster.sync();  // every block of the cluster runs, its weights and barriers are in place
-  uint32_t parity_a = 0, parity_w = 0;
-  bool alive = true;  // no wait has run out
+  uint32_t parity_a = 0;
+  bool late = false;  // a wait has run out
   // bytes of the weights that the other blocks send
   constexpr int kOwnTiles = 16 * (S::RS1 + S::RS2);
   const int w_bytes = 4 * ((NC - 1) * kOwnTiles + (bq == 0 ? 3 : 4) * 32 + (bq == 1 ? 3 : 4) * 16 + (rank == 1 ? 0 : 4));
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
         }
       }
       read_x();  // the next chunk's inputs arrive while the gradients run
-      if (alive) alive = tr_wait(bar_a, parity_a);
+      if (!late) late = !tr_wait(bar_a, parity_a);
       parity_a ^= 1;
       // ---- gradients, in sample order ---------------------------------------
       if (role < 2) {
@@ -540,15 +540,14 @@ __global__ void __launch_bounds__(TrainShape<NC>::T) mlp_train_kernel(const __gr
             tr_copy(d, v, v, bq == 0 ? 16 : 4, bar_w);
           }
         }
-        if (alive) alive = tr_wait(bar_w, parity_w);
-        parity_w ^= 1;
+        if (!late) late = !tr_wait(bar_w, (uint32_t)step & 1u);
       } else if (!last) {
         cluster.sync();  // everything read before it is overwritten
       }
     }
   }
   cluster.sync();  // no block leaves while another copies from or to it
-  if (!alive && p.status) set_status(p.status, GA_ERR_CUDA);
+  if (late && p.status) set_status(p.status, GA_ERR_CUDA);
   if (bad_idx && p.status) set_status(p.status, GA_ERR_ARG);
   if (upd)
     for (int e = 0; e < 4; ++e)
