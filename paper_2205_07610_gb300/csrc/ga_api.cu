@@ -2592,7 +2592,10 @@ int ga_align_cross(const uint8_t *q_codes, const int64_t *q_off, int64_t nq, con
   if ((rc = setup_sort(c))) return rc;
   SetView Q{q_codes, q_off, nullptr, nullptr}, T{t_codes, t_off, nullptr, nullptr};
   if ((rc = prepare_sets(c, Q, nq, T, nt))) return rc;
-  const int64_t kChunk = 1 << 22;
+  // Pairs planned at a time.  Alphabets of more than 4 symbols run as strips, whose
+  // edges for 4M protein pairs pass the limit of kx_prepare (90 queries x 40,000
+  // targets, global: 507 ms on the int32 kernel that then takes them, 201 ms so).
+  const int64_t kChunk = c.dna ? 1 << 22 : 1 << 20;
   const int64_t qpc = std::max<int64_t>(1, std::min<int64_t>(nq, kChunk / nt));
   const int64_t cap = qpc * nt;
   if (cap >= (1ll << 31) - 64) return GA_ERR_ARG;

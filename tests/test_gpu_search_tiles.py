@@ -69,3 +69,18 @@ def test_long_targets_beside_many_short_ones(nq, long_targets):
         got, st = ga.align_cross(*dev, mat, 11, 1, "local", stats=True)
         assert np.array_equal(got.cpu().numpy(), want)
         assert st["pairs_int16"] == nq * (len(ts) - bad) and (st["status"] != 0) == bad
+
+
+@pytest.mark.parametrize("mode", ["global", "semiglobal"])
+def test_more_pairs_than_one_plan_holds(mode):
+    # protein searches in the whole-sequence modes are planned 2^20 pairs at a time
+    rng = np.random.default_rng(6)
+    mat = synth.blosum62()
+    qs = [rng.integers(0, 20, size=int(n)).astype(np.uint8) for n in rng.integers(0, 8, size=1100)]
+    ts = [rng.integers(0, 20, size=int(n)).astype(np.uint8) for n in rng.integers(0, 8, size=1000)]
+    qc, qo = synth.pack_csr(qs)
+    tc, to = synth.pack_csr(ts)
+    dev = [torch.from_numpy(a).cuda() for a in (qc, qo, tc, to)]
+    want, _ = oracle.cross(qc, qo, tc, to, mat, 11, 1, mode, nthreads=NTHREADS)
+    got = ga.align_cross(*dev, mat, 11, 1, mode)
+    assert np.array_equal(got.cpu().numpy().ravel(), np.asarray(want).ravel())
