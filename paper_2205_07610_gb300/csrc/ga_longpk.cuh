@@ -42,6 +42,17 @@
 // Eq. H with nu = 0.  The running maximum is kept relative and folded into
 // an int32 maximum at every renormalisation.
 //
+// Semi-global mode: the last column's gap open is 0, so H(., C) keeps the largest
+// value of its column while the columns to its left may fall by beta a row: the
+// one place where neighbours can part further than above.  Nothing but E(., C)
+// reads H(., C), and a gap down a column whose end is free never beats stopping
+// there.  So at every renormalisation that value is folded into the int32 row
+// maximum and H and E of the column start again from the gap out of the column
+// beside it (pk_drop_free_end); until then they stay within the drift of the
+// column beside it.  Pad columns to the right may still see the old value and
+// wrap; they feed no real column, and lane-halves that hold nothing else get a base
+// below any score, so that the row maximum leaves them out.
+//
 // Rows outside a half's range: before its first row the high half sees a
 // "virtual" row whose table word leaves the row-0 state unchanged (sigma = 0
 // for local / semi-global; -beta for global, where H(0, j) = H(0, j-1) -
@@ -89,8 +100,37 @@ __device__ __forceinline__ uint32_t pk_row(uint32_t (&H)[K], uint32_t (&E)[K], u
   return F;
 }
 
+// Renormalisation, semi-global mode: folds H of the last column, `last` columns
+// after the lane's first of the low half (WH: columns of a half), into the row
+// maximum and drops its running value, also from the lane's pad columns beside it.
+constexpr int kPadBase = -(1 << 30);
+template <int K>
+__device__ __forceinline__ int pk_drop_free_end(uint32_t (&H)[K], uint32_t (&E)[K], uint32_t Hdiag, uint32_t NAc,
+                                                int last, int WH, int (&b)[2], int rowmax) {
+  const bool high = last >= WH;
+  const int at = high ? last - WH : last;
+  const uint32_t half = high ? 0xffff0000u : 0xffffu;
+  uint32_t x = 0;
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    if (j == at) {
+      rowmax = ::max(rowmax, high ? hi16(H[j]) + b[1] : lo16(H[j]) + b[0]);
+      x = __vadd2(j ? H[j - 1] : Hdiag, NAc) & half;
+    }
+    if (j >= at) {
+      H[j] = (H[j] & ~half) | x;
+      E[j] = (E[j] & ~half) | x;
+    }
+  }
+  if (last < 0) b[0] = kPadBase;
+  if (last < WH) b[1] = kPadBase;
+  return rowmax;
+}
+
+// (semi-global mode, 3,000 pairs of 1,000..2,000 residues in a plan, GB300: 2.26 ms with
+// three blocks per SM stated, 2.29 without, 2.44 with four)
 template <int MODE, int K>
-__global__ void __launch_bounds__(128) kw_kernel(const __grid_constant__ KBParams p) {
+__global__ void __launch_bounds__(128, MODE == kModeSemi ? 3 : 0) kw_kernel(const __grid_constant__ KBParams p) {
   static_assert(kKwMaxStep * (kKwRenorm + 2 * K + 8) < 32000 - 256, "relative int16 cells of this tile width");
   constexpr int kWarps = 4;
   constexpr int WH = 32 * K;  // columns per half
@@ -318,6 +358,8 @@ __global__ void __launch_bounds__(128) kw_kernel(const __grid_constant__ KBParam
           flushed = it0 - 63;
         }
         if ((it0 & (kKwRenorm - 1)) == 0 && it0 > 0) {
+          if constexpr (MODE == kModeSemi)
+            if (s == nst - 1) rowmax = pk_drop_free_end<K>(H, E, Hdiag, NAc, C - 1 - col0 - t * K, WH, b, rowmax);
           // move each half's base to its current H of the first column
           const int d0 = lo16(H[0]), d1 = hi16(H[0]);
           if constexpr (MODE == kModeLocal) {

@@ -39,6 +39,8 @@
 // exceed the largest real cell.  The loop ends when the last real column has
 // run its last row, so global mode's H(R, C) is what its owner holds then.
 //
+// Last column of semi-global mode: see ga_longpk.cuh.
+//
 // Edges.  The right edge of a strip (H and the outgoing F per row) goes to the
 // next strip through one 8-byte word per row in global memory: H (32 bits),
 // H - F (16 bits; alpha >= H - F >= beta), and the number of the strip that
@@ -346,6 +348,8 @@ __device__ __forceinline__ int kx_strip(const KXView &v, int s, int t, uint2 *ri
       on_rows(it0 - 63);
     }
     if ((it0 & (kKwRenorm - 1)) == 0 && it0 > 0) {
+      if constexpr (MODE == kModeSemi)
+        if (!edge_out) rowmax = pk_drop_free_end<K>(st.H, st.E, st.Hdiag, NAc, ncol - 1 - t * K, WH, b, rowmax);
       // move each half's base to its current H of the first column
       const int d0 = lo16(st.H[0]), d1 = hi16(st.H[0]);
       if constexpr (MODE == kModeLocal) {
