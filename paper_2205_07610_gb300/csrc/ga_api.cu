@@ -552,6 +552,8 @@ KXTaskScratch *kx_scratch(char *zero, int64_t n) {
   return reinterpret_cast<KXTaskScratch *>(zero + sizeof(KXPairState) * (size_t)n + 16);
 }
 
+constexpr int64_t kKxMaxEdgeWords = (4ll << 30) / 8;
+
 // Strip launch of a plan's long class: the task list and the zeroed edge words,
 // one buffer of (shorter sequence + 1) words per pair.  Left to the kernels that
 // run a pair on one warp where the relative int16 cells of the scoring are not
@@ -561,10 +563,10 @@ int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   if (std::max(c.sc.smax, 0) + c.sc.alpha > kKxMaxStep) return GA_OK;
   const LongSums &ls = p.r.long_sums;
   int64_t strips[kKxWidths];
-  for (int w = 0; w < kKxWidths; ++w) strips[w] = ls.strips[w];
+  for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)ls.strips[w];
   const int tile = kx_choose(p.mode, !c.dna, p.r.rmax_long, strips, c.nsm);
   const int64_t W = 64 * kKxTileK[tile], ntasks = strips[kKxTileK[tile] / 4 - 1];
-  if (p.r.rmax_long > W * kKxMaxStrips || ntasks > (1 << 30) || ls.rows > (4ull << 30) / 8) return GA_OK;
+  if (!kx_fits(tile, p.r.rmax_long, ntasks, (int64_t)ls.rows, kKxMaxEdgeWords)) return GA_OK;
   const int64_t cnt = p.long_cnt;
   const size_t head = kx_zeroed(cnt), bytes = head + 8 * (size_t)ls.rows;
   char *zero = c.al.try_get<char>(bytes);
@@ -1285,11 +1287,10 @@ struct BandRun {
   // Workspace, sized for every pair; without it every pair stays on the band kernel.
   int full_setup(Full &f) {
     int64_t strips[kKxWidths];
-    for (int w = 0; w < kKxWidths; ++w) strips[w] = sums.strips[w];
+    for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)sums.strips[w];
     f.tile = kx_choose(GA_GLOBAL, false, longest, strips, c.nsm);
-    const int64_t W = 64 * kKxTileK[f.tile];
-    if (longest > W * kKxMaxStrips || sums.rows > (4ull << 30) / 8) return GA_OK;
     f.cap = strips[kKxTileK[f.tile] / 4 - 1];
+    if (!kx_fits(f.tile, longest, f.cap, (int64_t)sums.rows, kKxMaxEdgeWords)) return GA_OK;
     f.bytes = kx_zeroed(npairs) + 8 * (size_t)sums.rows;
     f.zero = c.al.try_get<char>(f.bytes);
     if (f.zero) f.tasks = c.al.try_get<int2>((size_t)f.cap);
@@ -1589,7 +1590,7 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
       if (r > 0) {
         tile = kx_choose(GA_LOCAL, true, longest, strips, c.nsm, &kx);
         kx += 15e3 + 1.0 * r * nq;
-        if (longest > 64 * kKxTileK[tile] * kKxMaxStrips || rows > (1ll << 30) / 8) return;
+        if (!kx_fits(tile, longest, strips[kKxTileK[tile] / 4 - 1], rows, (1ll << 30) / 8)) return;
       }
       const bool none_left = n < 0 || (r < kKpTop && n == 0);
       const double warps = std::min(3.0, std::max(1.0, rest * nq / 4.0 / std::max<int64_t>(n, 1) / sched));

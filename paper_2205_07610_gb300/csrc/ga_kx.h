@@ -18,6 +18,23 @@ constexpr __host__ __device__ int kx_width(int w) { return 256 * (w + 1); }
 enum KxTile { kKx4 = 0, kKx8, kKx12, kKx16, kKx20, kKx8Wide, kKx16Wide, kKxTiles };
 constexpr int kKxTileK[kKxTiles] = {4, 8, 12, 16, 20, 8, 16};
 
+constexpr int kKxMaxStrips = 1024;         // strips of one pair (the task order's buckets)
+constexpr int64_t kKxMaxTasks = 1 << 30;   // strips of one launch (int32 places in its task list)
+
+// Sizes of a strip launch over a set of pairs: sum of (shorter sequence + 1), and the
+// strips of every width.  64 bits each: a search of one query of 200,000 residues
+// against 11 million targets has 8.6e9 strips of 256 columns.
+struct LongSums {
+  unsigned long long rows;
+  unsigned long long strips[kKxWidths];
+};
+
+// Whether a strip launch of a tile takes these sizes: the strips of the longest
+// sequence, all strips, and edge words of max_words at most.
+inline bool kx_fits(int tile, int64_t longest, int64_t ntasks, int64_t words, int64_t max_words) {
+  return longest <= 64 * (int64_t)kKxTileK[tile] * kKxMaxStrips && ntasks <= kKxMaxTasks && words <= max_words;
+}
+
 // The tile of a launch with strips[w] strips at width w whose longest pair has
 // `longest` rows: the one with the least estimated time.
 //

@@ -31,13 +31,6 @@ struct BinTable {
   int w32[kBins];
 };
 
-// Sizes of the strip launch over the long-class pairs (ga_strip.cuh): sum of
-// (shorter sequence + 1), and the strips of every width.
-struct LongSums {
-  unsigned long long rows;
-  int32_t strips[kKxWidths], pad;
-};
-
 struct PlanParams {
   const int64_t *q_off;
   const int64_t *t_off;
@@ -229,7 +222,7 @@ __device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongS
   unsigned long long rows = long_len ? (unsigned long long)short_len + 1 : 0;
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, off);
-  unsigned strips[kKxWidths];
+  unsigned strips[kKxWidths];  // (32 x 2^30 / 256 at most)
 #pragma unroll
   for (int w = 0; w < kKxWidths; ++w)
     strips[w] = __reduce_add_sync(0xffffffffu, ((unsigned)long_len + kx_width(w) - 1) / kx_width(w));
@@ -237,7 +230,7 @@ __device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongS
     atomicMax(longest, (int)cmax);
     atomicAdd(&sums->rows, rows);
 #pragma unroll
-    for (int w = 0; w < kKxWidths; ++w) atomicAdd(&sums->strips[w], (int)strips[w]);
+    for (int w = 0; w < kKxWidths; ++w) atomicAdd(&sums->strips[w], (unsigned long long)strips[w]);
   }
 }
 

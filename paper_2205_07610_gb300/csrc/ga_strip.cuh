@@ -60,13 +60,13 @@
 #pragma once
 
 #include "ga_dp.cuh"
+#include "ga_kx.h"
 #include "ga_longpk.cuh"
 
 namespace ga {
 
 constexpr int kKxWarps = 4;
 constexpr int kKxMaxStep = 128;       // largest sigma_max + alpha (relative int16 cells)
-constexpr int kKxMaxStrips = 1024;    // strips of one pair (the task order's buckets)
 constexpr int kKxRing = 64;           // row entries (+ a mirror of the first 34)
 constexpr int kKxSigRow = 9;          // words of a score vector in shared memory (32 bytes, odd stride)
 constexpr int64_t kKxWaitNs = 10ll * 1000 * 1000 * 1000;
