@@ -91,7 +91,9 @@ struct TrainParams {
 // barriers, the exchanges took 7 us: 13.8 us a step.)  The two waits order
 // everything: a block sends activations only after it has every block's weights,
 // and weights only after it has every block's activations, so what is overwritten
-// has been read; chunks without new weights end in a cluster barrier instead.  The
+// has been read, and no piece of a step is counted in the phase of another.  That
+// takes a piece from every block: one that holds no sample of a chunk sends 16 bytes
+// that nobody reads.  Chunks without new weights end in a cluster barrier instead.  The
 // next chunk's inputs are loaded a chunk ahead.  The last warp takes the biases,
 // the head and the loss.
 constexpr int kTrChunk = 256;  // samples per chunk
@@ -119,7 +121,8 @@ struct TrainShape {
   // what it receives, a row per sample of the chunk
   static constexpr int oD2 = oSR + SP, oD1 = oD2 + 16 * kTrChunk,
                        oH2 = oD1 + 16 * kTrChunk, oH1 = oH2 + 16 * kTrChunk, oX = oH1 + I2 * kTrChunk,
-                       oDY = oX + I1 * kTrChunk, oR = oDY + kTrChunk, oBar = oR + kTrChunk, kFloats = oBar + 4;
+                       oDY = oX + I1 * kTrChunk, oR = oDY + kTrChunk, oBar = oR + kTrChunk, oUnread = oBar + 4,
+                       kFloats = oUnread + 4;
   static_assert(oW2 % 4 == 0 && oB1 % 4 == 0 && kWeights % 4 == 0 && GS % 4 == 0 && GS1 % 4 == 0 && oBar % 4 == 0,
                 "16-byte pieces");
   static constexpr __device__ __forceinline__ int w1(int o, int i) {
@@ -332,6 +335,13 @@ __global__ void __launch_bounds__(TrainShape<NC>::T, 1) mlp_train_kernel(const _
   constexpr int kOwnTiles = 16 * (S::RS1 + S::RS2);
   const int w_bytes = 4 * ((NC - 1) * kOwnTiles + (bq == 0 ? 3 : 4) * 32 + (bq == 1 ? 3 : 4) * 16 + (rank == 1 ? 0 : 4));
 
+  // bytes of a chunk's activations: of a full one, of the rest
+  const int row_bytes = 4 * (S::I2 + 32 + (bq == 0 ? 17 : 0) + (rank == 1 ? 2 : 0));
+  const int rest = p.B % kTrChunk, rest_spc = ((rest + NC - 1) / NC + 3) & ~3;
+  const int a_bytes_full = row_bytes * kTrChunk;
+  const int a_bytes_rest =
+      rest ? row_bytes * ((rest + 3) & ~3) + 16 * (NC - (rest + rest_spc - 1) / rest_spc) : 0;
+
   for (int step = 0; step < p.steps; ++step) {
     if (upd && tid == 0) tr_expect(bar_w, w_bytes);
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -339,10 +349,7 @@ __global__ void __launch_bounds__(TrainShape<NC>::T, 1) mlp_train_kernel(const _
     for (int c0 = 0; c0 < p.B; c0 += kTrChunk) {
       const int cb = ::min(kTrChunk, p.B - c0);
       const int sb = own_base(cb);
-      if (tid == 0) {
-        const int rows = (cb + 3) & ~3;
-        tr_expect(bar_a, 4 * rows * (S::I2 + 32 + (bq == 0 ? 17 : 0) + (rank == 1 ? 2 : 0)));
-      }
+      if (tid == 0) tr_expect(bar_a, cb == kTrChunk ? a_bytes_full : a_bytes_rest);
       // ---- forward and backward of this warp's four samples -----------------
 #pragma unroll
       for (int j = 0; j < S::PER; ++j)
@@ -458,6 +465,8 @@ __global__ void __launch_bounds__(TrainShape<NC>::T, 1) mlp_train_kernel(const _
               tr_copy(d, tr_smem + S::oR + b0, tr_smem + S::oSR, n, bar_a);
             }
           }
+        } else if (warp == 0 && l < NC) {
+          tr_copy(l, tr_smem + S::oUnread, tr_smem + S::oSY, 4, bar_a);
         }
       }
       read_x();  // the next chunk's inputs arrive while the gradients run
