@@ -85,6 +85,8 @@ int ga_mlp_forward(const uint16_t *params_bf16, const float *x, int64_t n, float
  * samples (x: float32[n*32], target: float32[n]) and its gradient with
  * respect to the bf16 weights, grad: float32[6337] (same layout), loss:
  * float32[1] or NULL.  Batch sums run in sample order (deterministic).
+ * Does not synchronise; a value whose inputs did not arrive within the
+ * kernel's limit of seconds is NaN.
  */
 int ga_mlp_loss_grad(const uint16_t *params_bf16, const float *x, const float *target, int32_t n,
                      float *grad, float *loss, void *stream);
@@ -99,7 +101,8 @@ int ga_mlp_loss_grad(const uint16_t *params_bf16, const float *x, const float *t
  * uses step numbers step0+1 .. step0+steps.  losses: device
  * float32[steps] or NULL, the loss of each minibatch.  All steps run in one
  * kernel launch.  Synchronises the stream; GA_ERR_ARG also when a batch index is out of
- * range.
+ * range, GA_ERR_CUDA also when a wait of the kernel ran out (the parameters
+ * are not valid then).
  */
 int ga_mlp_train(float *master, uint16_t *params_bf16, float *adam_m, float *adam_v, const float *x,
                  const float *target, int64_t nsamples, const int32_t *batch_idx, int32_t steps,

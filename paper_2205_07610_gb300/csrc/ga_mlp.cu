@@ -514,10 +514,10 @@ __global__ void __launch_bounds__(TrainShape<NC>::T, 1) mlp_train_kernel(const _
         for (int b = 0; b < cb; ++b) acc[0] = fmaf(pu[b * su], sum_only ? 1.f : pv[b * sv], acc[0]);
       }
       if (last) {
-        if (is_loss && p.loss_out) p.loss_out[step] = 0.5f * acc[0] / (float)p.B;
+        if (is_loss && p.loss_out) p.loss_out[step] = late ? NAN : 0.5f * acc[0] / (float)p.B;
         if (p.grad_out)
           for (int e = 0; e < 4; ++e)
-            if (par[e] >= 0) p.grad_out[par[e]] = acc[e];
+            if (par[e] >= 0) p.grad_out[par[e]] = late ? NAN : acc[e];  // (no status to set)
         if (upd && role < 2) {
           float n[4];
 #pragma unroll
