@@ -484,8 +484,14 @@ __global__ void __launch_bounds__(32 * kSvWarps, 4) ks_kernel(const __grid_const
               const unsigned long long h = atomicAdd(&ctl->cont_head.v, 1ull);
               const int64_t e = (int64_t)(h % (unsigned long long)p.cont_cap);
               // (as many entries are published as tickets were drawn, but entry h
-              // may be one whose warp is between reserving and publishing it)
-              while (sv_ld_acquire64(p.cont_seq + e) != h + 1 && sv_now() - now < (uint64_t)p.wait_ns) {
+              // may be one whose warp is between reserving and publishing it; one that
+              // never shows is not read: the warp leaves, its request stays open)
+              bool there;
+              while (!(there = sv_ld_acquire64(p.cont_seq + e) == h + 1) && sv_now() - now < (uint64_t)p.wait_ns) {
+              }
+              if (!there) {
+                quit = 1;
+                break;
               }
               const int2 tk = __ldcg(p.cont + e);
               slot = tk.x;
