@@ -555,10 +555,11 @@ KXTaskScratch *kx_scratch(char *zero, int64_t n) {
 constexpr int64_t kKxMaxEdgeWords = (4ll << 30) / 8;
 
 // Strip launch of a plan's long class: the task list and the zeroed edge words,
-// one buffer of (shorter sequence + 1) words per pair.  Left to the kernels that
+// one buffer of (shorter sequence + 1) words per pair of more than one strip, in one
+// allocation.  Left to the kernels that
 // run a pair on one warp where the relative int16 cells of the scoring are not
 // exact, a pair has too many strips, or the edges would take more than 4 GB.
-int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
+int kx_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPlan &p) {
   p.kx_tile = -1;
   if (std::max(c.sc.smax, 0) + c.sc.alpha > kKxMaxStep) return GA_OK;
   const LongSums &ls = p.r.long_sums;
@@ -566,13 +567,14 @@ int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)ls.strips[w];
   const int tile = kx_choose(p.mode, !c.dna, p.r.rmax_long, strips, c.nsm);
   const int64_t W = 64 * kKxTileK[tile], ntasks = strips[kKxTileK[tile] / 4 - 1];
-  if (!kx_fits(tile, p.r.rmax_long, ntasks, (int64_t)ls.rows, kKxMaxEdgeWords)) return GA_OK;
+  const int64_t words = (int64_t)ls.words[kKxTileK[tile] / 4 - 1];
+  if (!kx_fits(tile, p.r.rmax_long, ntasks, words, kKxMaxEdgeWords)) return GA_OK;
   const int64_t cnt = p.long_cnt;
-  const size_t head = kx_zeroed(cnt), bytes = head + 8 * (size_t)ls.rows;
-  char *zero = c.al.try_get<char>(bytes);
-  int2 *tasks = zero ? c.al.try_get<int2>((size_t)ntasks) : nullptr;
-  int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)cnt) : nullptr;
-  if (!edge_off) return GA_OK;
+  const size_t head = kx_zeroed(cnt), bytes = head + 8 * (size_t)words;
+  char *zero = work.try_get<char>(bytes + sizeof(int2) * (size_t)ntasks + sizeof(int64_t) * (size_t)cnt);
+  if (!zero) return GA_OK;
+  int2 *tasks = reinterpret_cast<int2 *>(zero + bytes);
+  int64_t *edge_off = reinterpret_cast<int64_t *>(tasks + ntasks);
   KXParams &k = p.kx;
   k = KXParams{};
   k.q_codes = Q.codes;
@@ -620,7 +622,7 @@ int kx_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
 
 // Launch count, long-class grid and edge buffer of a read-back plan.  The
 // buffer is allocated here, before the fork: the side streams start after it.
-int launch_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
+int launch_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPlan &p) {
   p.nlaunch = 0;
   p.counter = 0;
   if (p.npairs == 0) return GA_OK;
@@ -631,7 +633,7 @@ int launch_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
   const bool profile = !c.dna;
   p.long_smem = profile ? (size_t)kKbWarps * (size_t)(c.sc.A + 1) * (32 * kKbK) : 0;
   if (p.long_cnt > 0) {
-    if (int rc = kx_prepare(c, Q, T, p)) return rc;
+    if (int rc = kx_prepare(c, work, Q, T, p)) return rc;
     if (p.kx_tile >= 0) return GA_OK;
     int occ = 0;
     if (long_packed(c.sc, c.dna))
@@ -649,8 +651,8 @@ int launch_prepare(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
     const int64_t want = (p.long_cnt + kKbWarps - 1) / kKbWarps;
     p.long_grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)c.nsm * std::max(occ, 1)));
     p.long_stride = (int64_t)p.r.rmax_long + 128;
-    p.long_bnd = c.al.get<int2>((size_t)p.long_grid * kKbWarps * (size_t)p.long_stride);
-    if (c.al.failed) return GA_ERR_OOM;
+    p.long_bnd = work.get<int2>((size_t)p.long_grid * kKbWarps * (size_t)p.long_stride);
+    if (work.failed) return GA_ERR_OOM;
   }
   return GA_OK;
 }
@@ -833,11 +835,12 @@ int rerun_enqueue(Call &c, const SetView &Q, const SetView &T, ChunkPlan &p) {
 // mode) as one unit: nothing waits for the host between them.
 int run_plans(Call &c, const SetView &Q, const SetView &T, ChunkPlan *ps, int n) {
   int rc;
+  Alloc work(c.s);  // freed behind the join: the next chunk of a search takes the same memory
   for (int k = 0; k < n; ++k)
     if ((rc = plan_enqueue(c, Q, T, ps[k]))) return rc;
   if ((rc = plan_readback(c, ps, n))) return rc;
   for (int k = 0; k < n; ++k)
-    if ((rc = launch_prepare(c, Q, T, ps[k]))) return rc;
+    if ((rc = launch_prepare(c, work, Q, T, ps[k]))) return rc;
   if ((rc = launch_plans(c, Q, T, ps, n))) return rc;
   for (int k = 0; k < n; ++k)
     if ((rc = rerun_enqueue(c, Q, T, ps[k]))) return rc;
@@ -1290,8 +1293,9 @@ struct BandRun {
     for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)sums.strips[w];
     f.tile = kx_choose(GA_GLOBAL, false, longest, strips, c.nsm);
     f.cap = strips[kKxTileK[f.tile] / 4 - 1];
-    if (!kx_fits(f.tile, longest, f.cap, (int64_t)sums.rows, kKxMaxEdgeWords)) return GA_OK;
-    f.bytes = kx_zeroed(npairs) + 8 * (size_t)sums.rows;
+    const int64_t words = (int64_t)sums.words[kKxTileK[f.tile] / 4 - 1];
+    if (!kx_fits(f.tile, longest, f.cap, words, kKxMaxEdgeWords)) return GA_OK;
+    f.bytes = kx_zeroed(npairs) + 8 * (size_t)words;
     f.zero = c.al.try_get<char>(f.bytes);
     if (f.zero) f.tasks = c.al.try_get<int2>((size_t)f.cap);
     if (f.tasks) f.edge_off = c.al.try_get<int64_t>((size_t)npairs);

@@ -21,12 +21,14 @@ constexpr int kKxTileK[kKxTiles] = {4, 8, 12, 16, 20, 8, 16};
 constexpr int kKxMaxStrips = 1024;         // strips of one pair (the task order's buckets)
 constexpr int64_t kKxMaxTasks = 1 << 30;   // strips of one launch (int32 places in its task list)
 
-// Sizes of a strip launch over a set of pairs: sum of (shorter sequence + 1), and the
-// strips of every width.  64 bits each: a search of one query of 200,000 residues
-// against 11 million targets has 8.6e9 strips of 256 columns.
+// Sizes of a strip launch over a set of pairs: sum of (shorter sequence + 1), and for
+// every width the strips and the edge words (the same sum over the pairs of more than
+// one strip).  64 bits each: a search of one query of 200,000 residues against 11
+// million targets has 8.6e9 strips of 256 columns.
 struct LongSums {
   unsigned long long rows;
   unsigned long long strips[kKxWidths];
+  unsigned long long words[kKxWidths];
 };
 
 // Whether a strip launch of a tile takes these sizes: the strips of the longest

@@ -214,24 +214,38 @@ __device__ __forceinline__ int global_gap(int alpha, int beta, int64_t len) {
   return len == 0 ? 0 : -(int)(alpha + beta * (len - 1));
 }
 
-// Adds the pairs of a warp (shorter and longer sequence; 0: none) to the sizes of
-// a strip launch.
+// Adds the pairs of a block (shorter and longer sequence; 0: none) to the sizes of a
+// strip launch: in a warp by reductions, in the block in shared memory, one atomic per
+// block and size.  Every thread of the block calls it.
 __device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongSums *sums, int32_t *longest) {
-  const unsigned cmax = __reduce_max_sync(0xffffffffu, (unsigned)long_len);
-  // 32 x (2^30 + 1) needs more than 32 bits
-  unsigned long long rows = long_len ? (unsigned long long)short_len + 1 : 0;
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ unsigned long long acc[1 + 2 * kKxWidths];  // as LongSums
+  __shared__ int cmax_s;
+  static_assert(sizeof(LongSums) == sizeof(acc), "one word per size");
+  if (!__syncthreads_or(long_len != 0)) return;
+  if (threadIdx.x < 1 + 2 * kKxWidths) acc[threadIdx.x] = 0;
+  if (threadIdx.x == 0) cmax_s = 0;
+  __syncthreads();
+  const unsigned cmax = __reduce_max_sync(FULL, (unsigned)long_len);
+  if (cmax) {
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    auto add = [&](int k, unsigned v) {  // (32 values of up to 2^30 + 1 need more than 32 bits)
+      const unsigned lo = __reduce_add_sync(FULL, v & 0xffffu), hi = __reduce_add_sync(FULL, v >> 16);
+      if (lane0 && (lo | hi)) atomicAdd(&acc[k], ((unsigned long long)hi << 16) + lo);
+    };
+    const unsigned rows = long_len ? (unsigned)short_len + 1 : 0;
+    add(0, rows);
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) rows += __shfl_xor_sync(0xffffffffu, rows, off);
-  unsigned strips[kKxWidths];  // (32 x 2^30 / 256 at most)
-#pragma unroll
-  for (int w = 0; w < kKxWidths; ++w)
-    strips[w] = __reduce_add_sync(0xffffffffu, ((unsigned)long_len + kx_width(w) - 1) / kx_width(w));
-  if ((threadIdx.x & 31) == 0 && cmax) {
-    atomicMax(longest, (int)cmax);
-    atomicAdd(&sums->rows, rows);
-#pragma unroll
-    for (int w = 0; w < kKxWidths; ++w) atomicAdd(&sums->strips[w], (unsigned long long)strips[w]);
+    for (int w = 0; w < kKxWidths; ++w) {
+      add(1 + w, ((unsigned)long_len + kx_width(w) - 1) / kx_width(w));
+      add(1 + kKxWidths + w, long_len > kx_width(w) ? rows : 0);
+    }
+    if (lane0) atomicMax(&cmax_s, (int)cmax);
   }
+  __syncthreads();
+  if (threadIdx.x < 1 + 2 * kKxWidths && acc[threadIdx.x])
+    atomicAdd(reinterpret_cast<unsigned long long *>(sums) + threadIdx.x, acc[threadIdx.x]);
+  if (threadIdx.x == 0) atomicMax(longest, cmax_s);
 }
 
 // One pair (batch) or (query, target) combination (cross chunk).
@@ -311,7 +325,7 @@ __global__ void plan_kernel(PlanParams p) {
   unsigned long long my_cells = 0;
   int long_rows = 0, long_cols = 0;
   if (i < p.npairs) plan_one(p, i, my_cells, long_rows, long_cols);
-  if (__any_sync(0xffffffffu, long_cols != 0)) add_long_sums(long_rows, long_cols, p.long_sums, p.rmax_long);
+  add_long_sums(long_rows, long_cols, p.long_sums, p.rmax_long);
   // one atomic per warp for the cell count
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) my_cells += __shfl_xor_sync(0xffffffffu, my_cells, off);
