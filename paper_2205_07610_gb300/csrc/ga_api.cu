@@ -1251,10 +1251,9 @@ struct BandRun {
     kc.bis_lo = bis_lo;
     kc.bis_hi = bis_hi;
     Full f;
-    if (packed && !bis_lo)
-      if (int rc = full_setup(f)) return rc;
-    if (f.on && full_first(default_w0, w0 != nullptr)) return full_run(f, kc, sorted, kc.range, nullptr);
-    f.on = f.on && few_pairs();
+    const bool first = packed && !bis_lo && full_first(default_w0, w0 != nullptr);
+    if (first || (packed && !bis_lo && few_pairs())) full_setup(f);
+    if (f.on && first) return full_run(f, kc, sorted, kc.range, nullptr);
     if (f.on) {
       kc.hand_count = &c.small->hand_range[1];
       kc.hand_list = f.list;
@@ -1287,24 +1286,26 @@ struct BandRun {
   // 117).
   bool few_pairs() const { return npairs <= 2 * (int64_t)c.nsm * std::max(blocks_per_sm_kz(), 1) * kKcWarps; }
 
-  // Workspace, sized for every pair; without it every pair stays on the band kernel.
-  int full_setup(Full &f) {
+  // Workspace, sized for every pair, for a call that uses it; without it every pair
+  // stays on the band kernel.
+  void full_setup(Full &f) {
     int64_t strips[kKxWidths];
     for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)sums.strips[w];
     f.tile = kx_choose(GA_GLOBAL, false, longest, strips, c.nsm);
     f.cap = strips[kKxTileK[f.tile] / 4 - 1];
     const int64_t words = (int64_t)sums.words[kKxTileK[f.tile] / 4 - 1];
-    if (!kx_fits(f.tile, longest, f.cap, words, kKxMaxEdgeWords)) return GA_OK;
+    if (!kx_fits(f.tile, longest, f.cap, words, kKxMaxEdgeWords)) return;
     f.bytes = kx_zeroed(npairs) + 8 * (size_t)words;
-    f.zero = c.al.try_get<char>(f.bytes);
-    if (f.zero) f.tasks = c.al.try_get<int2>((size_t)f.cap);
-    if (f.tasks) f.edge_off = c.al.try_get<int64_t>((size_t)npairs);
-    if (f.edge_off) f.list = c.al.try_get<int32_t>((size_t)npairs);
-    if (f.list) f.w_next = c.al.try_get<int32_t>((size_t)npairs);
-    if (f.w_next) f.tie_list = c.al.try_get<int32_t>((size_t)npairs);
-    if (f.tie_list) f.tie_w = c.al.try_get<int32_t>((size_t)npairs);
-    f.on = f.tie_w != nullptr;
-    return GA_OK;
+    f.zero = c.al.try_get<char>(f.bytes + sizeof(int2) * (size_t)f.cap +
+                                (sizeof(int64_t) + 4 * sizeof(int32_t)) * (size_t)npairs);
+    if (!f.zero) return;
+    f.tasks = reinterpret_cast<int2 *>(f.zero + f.bytes);
+    f.edge_off = reinterpret_cast<int64_t *>(f.tasks + f.cap);
+    f.list = reinterpret_cast<int32_t *>(f.edge_off + npairs);
+    f.w_next = f.list + npairs;
+    f.tie_list = f.w_next + npairs;
+    f.tie_w = f.tie_list + npairs;
+    f.on = true;
   }
 
   // Whether the full matrices of all pairs are the faster way, in cycles.  They
