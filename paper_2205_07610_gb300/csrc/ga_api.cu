@@ -172,9 +172,11 @@ struct Alloc {
     failed = was;
     return p;
   }
-  ~Alloc() {
+  void release() {
     for (void *p : ptrs) cudaFreeAsync(p, s);
+    ptrs.clear();
   }
+  ~Alloc() { release(); }
 };
 
 // Small pinned staging area for scalar readbacks (one per host thread).
@@ -1619,17 +1621,18 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
 
 // Task list and workspace of the chosen targets, on the call's stream; without the
 // workspace the search kernel keeps them.
-int kp_split_prepare(Call &c, const SetView &Q, const SetView &T, int64_t nt, const int32_t *queries, int64_t nqv,
-                     const int32_t *sorted, int32_t *scores, KpSplit &sp) {
+int kp_split_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, int64_t nt, const int32_t *queries,
+                     int64_t nqv, const int32_t *sorted, int32_t *scores, KpSplit &sp) {
   const size_t head = kx_zeroed(sp.npairs), bytes = head + 8 * (size_t)sp.rows;
-  char *zero = c.al.try_get<char>(bytes);
-  int2 *tasks = zero ? c.al.try_get<int2>((size_t)sp.strips) : nullptr;
-  int64_t *edge_off = tasks ? c.al.try_get<int64_t>((size_t)sp.npairs) : nullptr;
-  int32_t *list = edge_off ? c.al.try_get<int32_t>((size_t)sp.npairs) : nullptr;
-  if (!list) {
+  char *zero = work.try_get<char>(bytes + sizeof(int2) * (size_t)sp.strips +
+                                  (sizeof(int64_t) + sizeof(int32_t)) * (size_t)sp.npairs);
+  if (!zero) {
     sp.ntargets = 0;
     return GA_OK;
   }
+  int2 *tasks = reinterpret_cast<int2 *>(zero + bytes);
+  int64_t *edge_off = reinterpret_cast<int64_t *>(tasks + sp.strips);
+  int32_t *list = reinterpret_cast<int32_t *>(edge_off + sp.npairs);
   KXParams &k = sp.kx;
   k.q_codes = Q.codes;
   k.t_codes = T.codes;
@@ -1758,13 +1761,13 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
     return GA_ERR_CUDA;
   const int32_t ntv_all = ntv;
   KpSplit sp;
+  Alloc split_work(c.s);
   if (ntv > 0) {
     std::sort(qlen.begin(), qlen.end());
     kp_split_choose(c, qlen, top[0], max_len, sp);
     if (sp.ntargets &&
-        (rc = kp_split_prepare(c, Q, T, nt, dq, (int64_t)flat.size(), sorted, scores, sp)))
+        (rc = kp_split_prepare(c, split_work, Q, T, nt, dq, (int64_t)flat.size(), sorted, scores, sp)))
       return rc;
-    ntv -= sp.ntargets;
   }
   KPParams kp{};
   kp.q_codes = q_codes;
@@ -1772,8 +1775,6 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   kp.t_codes = t_codes;
   kp.t_packed5 = t_packed5;
   kp.t_off = t_off;
-  kp.t_sorted = sorted + sp.ntargets;
-  kp.ntv = ntv;
   kp.nt = nt;
   kp.A = c.sc.A;
   kp.alpha = c.sc.alpha;
@@ -1790,31 +1791,49 @@ int cross_protein_local(Call &c, const uint8_t *q_codes, const int64_t *q_off, i
   // queries x 2,000 targets 4.65 ms in order, 1.9 together).  The bins whose rows cost most come
   // first, so the last launch's longest target is a short chain.  Bins of several
   // stages keep their edges in a buffer of their own; where these would take more
-  // than 4 GB the launches run in order and share one.
+  // than 4 GB, or more than there is, the launches run in order and share one.  Where
+  // not even that one fits, the workspace of the split targets is given back first.
   KPParams kps[kKpTiles];
-  int grids[kKpTiles] = {}, order[kKpTiles], nlaunch = 0;
-  size_t edges[kKpTiles] = {}, edge_sum = 0, edge_max = 0, off = 0;
-  double chain[kKpTiles] = {};
-  for (int b = 0; b < kKpTiles; ++b) {
-    const int32_t *queries = dq + off;
-    off += bins[b].size();
-    if (bins[b].empty() || ntv == 0) continue;
-    kp.queries = queries;
-    kp.nqb = (int32_t)bins[b].size();
-    kp.task_counter = &c.small->counters[b];
-    const int64_t W = (int64_t)kKpG * kKpTileK[b], nst = (hqo[(size_t)bins[b][0] + 1] - hqo[(size_t)bins[b][0]] + W - 1) / W;
-    if ((grids[b] = kp_grid_tile(c, kp, b)) <= 0) return GA_ERR_CUDA;
-    if (nst > 1) edges[b] = (size_t)grids[b] * kKpGroups * (size_t)kp.bnd_stride;
-    edge_sum += edges[b];
-    edge_max = std::max(edge_max, edges[b]);
-    chain[b] = (double)(nst * W);
-    kps[b] = kp;
-    order[nlaunch++] = b;
+  int grids[kKpTiles], order[kKpTiles], nlaunch;
+  size_t edges[kKpTiles];
+  bool together;
+  int2 *bnd;
+  for (;;) {
+    size_t edge_sum = 0, edge_max = 0, off = 0;
+    double chain[kKpTiles] = {};
+    ntv = ntv_all - sp.ntargets;
+    kp.t_sorted = sorted + sp.ntargets;
+    kp.ntv = ntv;
+    nlaunch = 0;
+    for (int b = 0; b < kKpTiles; ++b) {
+      const int32_t *queries = dq + off;
+      off += bins[b].size();
+      if (bins[b].empty() || ntv == 0) continue;
+      kp.queries = queries;
+      kp.nqb = (int32_t)bins[b].size();
+      kp.task_counter = &c.small->counters[b];
+      const int64_t W = (int64_t)kKpG * kKpTileK[b], nst = (hqo[(size_t)bins[b][0] + 1] - hqo[(size_t)bins[b][0]] + W - 1) / W;
+      if ((grids[b] = kp_grid_tile(c, kp, b)) <= 0) return GA_ERR_CUDA;
+      edges[b] = nst > 1 ? (size_t)grids[b] * kKpGroups * (size_t)kp.bnd_stride : 0;
+      edge_sum += edges[b];
+      edge_max = std::max(edge_max, edges[b]);
+      chain[b] = (double)(nst * W);
+      kps[b] = kp;
+      order[nlaunch++] = b;
+    }
+    std::stable_sort(order, order + nlaunch, [&](int x, int y) { return chain[x] > chain[y]; });
+    bnd = nullptr;
+    together = edge_sum * sizeof(int2) <= (4ull << 30);
+    if (edge_max && together) bnd = c.al.try_get<int2>(edge_sum);
+    if (edge_max && !bnd) {
+      together = false;
+      bnd = c.al.try_get<int2>(edge_max);
+    }
+    if (bnd || !edge_max) break;
+    if (!sp.ntargets) return GA_ERR_OOM;
+    split_work.release();
+    sp = KpSplit();
   }
-  std::stable_sort(order, order + nlaunch, [&](int x, int y) { return chain[x] > chain[y]; });
-  const bool together = edge_sum * sizeof(int2) <= (4ull << 30);
-  int2 *bnd = edge_max ? c.al.get<int2>(together ? edge_sum : edge_max) : nullptr;
-  if (c.al.failed) return GA_ERR_OOM;
   {
     DpFork fk(c);
     const int nkx = sp.ntargets > 0;
