@@ -1477,11 +1477,14 @@ int features_impl(const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t
 // packed query-profile kernel: targets sorted longest first, queries binned
 // by length (columns per lane K = 8, 16, 24 or 32; longer queries run in
 // stages of 512 columns), flagged pairs recomputed exactly in int32.
+// (The kernels' shared-memory limit, one setting per device for every host thread, is
+// that of 31 symbols whatever the call's.)
 template <int K>
 int kp_grid(Call &c, const KPParams &kp) {
   const size_t smem = sizeof(uint32_t) * (size_t)kp_prof_words<K>(c.sc.A);
   int occ = 0;
-  if (cudaFuncSetAttribute(kp_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+  if (cudaFuncSetAttribute(kp_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(sizeof(uint32_t) * kp_prof_words<K>(31))) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp_kernel<K>, 32 * kKpWarps, smem) != cudaSuccess)
     return 0;
   const int64_t ntasks = (int64_t)((kp.nqb + 1) / 2) * ((kp.ntv + kKpGroups - 1) / kKpGroups);

@@ -6,12 +6,16 @@
 
 namespace ga {
 
+// (A kernel's shared-memory limit is one setting per device for every host thread: it
+// is set to the largest alphabet's profile, so that no call lowers it below what
+// another one is about to launch with.)
 template <int MODE, int K, bool FC, bool PROF>
 cudaError_t kx_launch(const KXParams &p, int grid, cudaStream_t s, int *occ) {
+  constexpr size_t largest = (size_t)kKxWarps * 32 * kx_prof_row<K>;
   const size_t smem = PROF ? (size_t)kKxWarps * (size_t)(p.A + 1) * kx_prof_row<K> : 0;
-  if (smem > 40 * 1024) {
+  if (PROF && largest > 40 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kx_kernel<MODE, K, FC, PROF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+                                               (int)largest);
     if (e != cudaSuccess) return e;
   }
   if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kx_kernel<MODE, K, FC, PROF>, 32 * kKxWarps, smem);

@@ -171,12 +171,14 @@ int blocks_per_sm_ka_alt_tile(int bin) {
   }                                                                                     \
   int blocks_per_sm_##NAME(int bin) { return blocks_per_sm_ka_alt_tile<MODE>(bin); }
 
+// (A kernel's shared-memory limit is one setting per device for every host thread: it
+// is set to the profile of the largest alphabet, 31 symbols, whatever the call's.)
 #define GA_KB_DEFINE(NAME, MODE, PROFILE)                                                    \
   cudaError_t launch_##NAME(const KBParams &p, int grid, size_t smem, cudaStream_t s) {     \
     if (smem > 48 * 1024) {                                                                  \
       cudaError_t e = cudaFuncSetAttribute(kb_kernel<MODE, kKbK, PROFILE>,                   \
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                           (int)smem);                                       \
+                                           kKbWarps * 32 * (32 * kKbK));                     \
       if (e != cudaSuccess) return e;                                                        \
     }                                                                                        \
     kb_kernel<MODE, kKbK, PROFILE><<<grid, kKbThreads, smem, s>>>(p);                        \
@@ -186,7 +188,8 @@ int blocks_per_sm_ka_alt_tile(int bin) {
     int n = 0;                                                                               \
     if (smem > 48 * 1024)                                                                    \
       cudaFuncSetAttribute(kb_kernel<MODE, kKbK, PROFILE>,                                   \
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);          \
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,                      \
+                           kKbWarps * 32 * (32 * kKbK));                                     \
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kb_kernel<MODE, kKbK, PROFILE>,        \
                                                   kKbThreads, smem);                         \
     return n;                                                                                \
