@@ -565,9 +565,12 @@ int kx_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPl
   p.kx_tile = -1;
   if (std::max(c.sc.smax, 0) + c.sc.alpha > kKxMaxStep) return GA_OK;
   const LongSums &ls = p.r.long_sums;
-  int64_t strips[kKxWidths];
-  for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)ls.strips[w];
-  const int tile = kx_choose(p.mode, !c.dna, p.r.rmax_long, strips, c.nsm);
+  int64_t strips[kKxWidths], chain[kKxWidths];
+  for (int w = 0; w < kKxWidths; ++w) {
+    strips[w] = (int64_t)ls.strips[w];
+    chain[w] = ls.chain[w];
+  }
+  const int tile = kx_choose(p.mode, !c.dna, chain, strips, c.nsm);
   const int64_t W = 64 * kKxTileK[tile], ntasks = strips[kKxTileK[tile] / 4 - 1];
   const int64_t words = (int64_t)ls.words[kKxTileK[tile] / 4 - 1];
   if (!kx_fits(tile, p.r.rmax_long, ntasks, words, kKxMaxEdgeWords)) return GA_OK;
@@ -1043,9 +1046,12 @@ int kx_align_pair(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, cons
       cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return GA_ERR_CUDA;
   const int64_t R = std::min(m, n), C = std::max(m, n);
-  int64_t strips[kKxWidths];
-  for (int w = 0; w < kKxWidths; ++w) strips[w] = (C + kx_width(w) - 1) / kx_width(w);
-  const int tile = kx_choose(mode, sc.A > 4, R, strips, c.nsm);
+  int64_t strips[kKxWidths], chain[kKxWidths];
+  for (int w = 0; w < kKxWidths; ++w) {
+    strips[w] = (C + kx_width(w) - 1) / kx_width(w);
+    chain[w] = kx_chain(R, C, w);
+  }
+  const int tile = kx_choose(mode, sc.A > 4, chain, strips, c.nsm);
   const int64_t ns = strips[kKxTileK[tile] / 4 - 1];
   const size_t head = sizeof(KXPairState) + 16, bytes = head + (ns > 1 ? 8 * (size_t)(R + 1) : 0);
   Events ev(stats != nullptr, s);
@@ -1291,9 +1297,12 @@ struct BandRun {
   // Workspace, sized for every pair, for a call that uses it; without it every pair
   // stays on the band kernel.
   void full_setup(Full &f) {
-    int64_t strips[kKxWidths];
-    for (int w = 0; w < kKxWidths; ++w) strips[w] = (int64_t)sums.strips[w];
-    f.tile = kx_choose(GA_GLOBAL, false, longest, strips, c.nsm);
+    int64_t strips[kKxWidths], chain[kKxWidths];
+    for (int w = 0; w < kKxWidths; ++w) {
+      strips[w] = (int64_t)sums.strips[w];
+      chain[w] = sums.chain[w];
+    }
+    f.tile = kx_choose(GA_GLOBAL, false, chain, strips, c.nsm);
     f.cap = strips[kKxTileK[f.tile] / 4 - 1];
     const int64_t words = (int64_t)sums.words[kKxTileK[f.tile] / 4 - 1];
     if (!kx_fits(f.tile, longest, f.cap, words, kKxMaxEdgeWords)) return;
@@ -1321,9 +1330,12 @@ struct BandRun {
   // 8.6 / 18.6, 1,500 34 / 13 / 31.6; from w = 64 1,500 34 / 26 / 55.
   bool full_first(int32_t default_w0, bool per_pair) const {
     double full = 0;
-    int64_t one[kKxWidths];
-    for (int w = 0; w < kKxWidths; ++w) one[w] = (longest + kx_width(w) - 1) / kx_width(w);
-    kx_choose(GA_GLOBAL, false, longest, one, c.nsm, &full);
+    int64_t one[kKxWidths], chain[kKxWidths];
+    for (int w = 0; w < kKxWidths; ++w) {
+      one[w] = (longest + kx_width(w) - 1) / kx_width(w);
+      chain[w] = sums.chain[w];
+    }
+    kx_choose(GA_GLOBAL, false, chain, one, c.nsm, &full);
     full = std::max(full, full_cells / 2850.0);
     const double rows = max_rows, stages = (double)(longest / kBandStageCols);
     // (widths given per pair: the average window, one attempt)
@@ -1589,7 +1601,7 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
     above[w].assign(nq + 1, 0);
     for (size_t k = nq; k-- > 0;) above[w][k] = above[w][k + 1] + (qlen[k] + kx_width(w) - 1) / kx_width(w);
   }
-  int64_t strips[kKxWidths] = {}, rows = 0;
+  int64_t strips[kKxWidths] = {}, chain[kKxWidths] = {}, rows = 0;
   double rest = (double)top.residues, best = 0;
   const int64_t longest = std::max(qlen[nq - 1], max_len);
   for (int r = 0; r <= kKpTop; ++r) {
@@ -1598,7 +1610,7 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
       double kx = 0;
       int tile = 0;
       if (r > 0) {
-        tile = kx_choose(GA_LOCAL, true, longest, strips, c.nsm, &kx);
+        tile = kx_choose(GA_LOCAL, true, chain, strips, c.nsm, &kx);
         kx += 15e3 + 1.0 * r * nq;
         if (!kx_fits(tile, longest, strips[kKxTileK[tile] / 4 - 1], rows, (1ll << 30) / 8)) return;
       }
@@ -1616,7 +1628,10 @@ void kp_split_choose(const Call &c, const std::vector<int64_t> &qlen /* ascendin
       if (none_left || r == kKpTop) return;
     }
     const size_t k = std::upper_bound(qlen.begin(), qlen.end(), n) - qlen.begin();  // queries up to n residues
-    for (int w = 0; w < kKxWidths; ++w) strips[w] += (int64_t)k * ((n + kx_width(w) - 1) / kx_width(w)) + above[w][k];
+    for (int w = 0; w < kKxWidths; ++w) {
+      strips[w] += (int64_t)k * ((n + kx_width(w) - 1) / kx_width(w)) + above[w][k];
+      chain[w] = std::max(chain[w], kx_chain(std::min(n, qlen[nq - 1]), std::max(n, qlen[nq - 1]), w));
+    }
     rows += below[k] + (int64_t)(nq - k) * n + (int64_t)nq;
     rest -= (double)n;
   }

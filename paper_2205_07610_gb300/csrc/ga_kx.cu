@@ -16,10 +16,9 @@ constexpr Step kSteps[4][kKxTiles] = {
     {{104, 52, 0}, {172, 84, 40}, {230, 105, 50}, {}, {}, {}, {290, 160, 60}},
     {{95, 66, 0}, {150, 114, 0}, {}, {}, {}, {175, 103, 20}, {}},
     {{104, 66, 0}, {175, 103, 20}, {}, {}, {}, {}, {}}};
-constexpr int kLag = 115;  // rows a strip runs behind its left neighbour
 }  // namespace
 
-int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, int nsm, double *cycles) {
+int kx_choose(int mode, bool profile, const int64_t *chain, const int64_t *strips, int nsm, double *cycles) {
   const Step *tab = kSteps[(profile ? 2 : 0) + (mode == 2 ? 1 : 0)];
   const int64_t sched = 4 * (int64_t)nsm;
   int best = -1;
@@ -28,7 +27,7 @@ int kx_choose(int mode, bool profile, int64_t longest, const int64_t *strips, in
     if (!tab[i].lone) continue;
     const int64_t n = strips[kKxTileK[i] / 4 - 1], w = (n + sched - 1) / sched;
     const double step = std::max<double>(tab[i].lone, (double)(w * tab[i].each + tab[i].fixed));
-    const double t = (double)(longest + kLag * (longest / (64 * kKxTileK[i]))) * step;
+    const double t = (double)chain[kKxTileK[i] / 4 - 1] * step;
     if (best < 0 || t < tbest) {
       best = i;
       tbest = t;

@@ -13,6 +13,8 @@
 //     starts first.
 #pragma once
 
+#include <cstddef>
+
 #include "ga_common.cuh"
 #include "ga_kx.h"
 
@@ -216,14 +218,15 @@ __device__ __forceinline__ int global_gap(int alpha, int beta, int64_t len) {
 
 // Adds the pairs of a block (shorter and longer sequence; 0: none) to the sizes of a
 // strip launch: in a warp by reductions, in the block in shared memory, one atomic per
-// block and size.  Every thread of the block calls it.
+// block and size.  (The chain of a pair of 2^30 residues stays below 2^31.)  Every thread of the block calls it.
 __device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongSums *sums, int32_t *longest) {
   constexpr unsigned FULL = 0xffffffffu;
-  __shared__ unsigned long long acc[1 + 2 * kKxWidths];  // as LongSums
-  __shared__ int cmax_s;
-  static_assert(sizeof(LongSums) == sizeof(acc), "one word per size");
+  __shared__ unsigned long long acc[1 + 2 * kKxWidths];  // as LongSums up to chain
+  __shared__ int chain_s[kKxWidths], cmax_s;
+  static_assert(offsetof(LongSums, chain) == sizeof(acc), "one word per sum");
   if (!__syncthreads_or(long_len != 0)) return;
   if (threadIdx.x < 1 + 2 * kKxWidths) acc[threadIdx.x] = 0;
+  if (threadIdx.x < kKxWidths) chain_s[threadIdx.x] = 0;
   if (threadIdx.x == 0) cmax_s = 0;
   __syncthreads();
   const unsigned cmax = __reduce_max_sync(FULL, (unsigned)long_len);
@@ -239,12 +242,15 @@ __device__ __forceinline__ void add_long_sums(int short_len, int long_len, LongS
     for (int w = 0; w < kKxWidths; ++w) {
       add(1 + w, ((unsigned)long_len + kx_width(w) - 1) / kx_width(w));
       add(1 + kKxWidths + w, long_len > kx_width(w) ? rows : 0);
+      const unsigned chain = __reduce_max_sync(FULL, (unsigned)kx_chain(short_len, long_len, w));
+      if (lane0) atomicMax(&chain_s[w], (int)chain);
     }
     if (lane0) atomicMax(&cmax_s, (int)cmax);
   }
   __syncthreads();
   if (threadIdx.x < 1 + 2 * kKxWidths && acc[threadIdx.x])
     atomicAdd(reinterpret_cast<unsigned long long *>(sums) + threadIdx.x, acc[threadIdx.x]);
+  if (threadIdx.x < kKxWidths) atomicMax(&sums->chain[threadIdx.x], chain_s[threadIdx.x]);
   if (threadIdx.x == 0) atomicMax(longest, cmax_s);
 }
 

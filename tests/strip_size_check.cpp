@@ -25,17 +25,18 @@ int main() {
   for (int k = 0; k < 5; ++k) {
     const Search &c = cases[k];
     LongSums s{};
-    int64_t strips[kKxWidths];
+    int64_t strips[kKxWidths], chain[kKxWidths];
     for (int w = 0; w < kKxWidths; ++w) {
       s.strips[w] += (unsigned long long)c.pairs * (unsigned long long)((c.longer + kx_width(w) - 1) / kx_width(w));
       strips[w] = (int64_t)s.strips[w];
+      chain[w] = kx_chain(c.shorter, c.longer, w);
       check(strips[w] / c.pairs == (c.longer + kx_width(w) - 1) / kx_width(w), "strip totals are not cut off");
     }
     check(kx_fits(kKx4, c.longer, strips[0], c.pairs * (c.shorter + 1), (4ll << 30) / 8) == fits4[k],
           "a launch of 256-column strips");
     for (const bool profile : {false, true})
       for (int mode = 0; mode < 3; ++mode) {
-        const int tile = kx_choose(mode, profile, c.longer, strips, 152);
+        const int tile = kx_choose(mode, profile, chain, strips, 152);
         const int64_t n = strips[kKxTileK[tile] / 4 - 1];
         check(!kx_fits(tile, c.longer, n, 0, 1) || n <= kKxMaxTasks, "the chosen tile's tasks");
       }
