@@ -77,9 +77,11 @@ extern "C" {
  * fill of every pair at the cost of more registers per lane, more lanes do
  * the opposite.  concurrent = 1 runs the bins as parallel branches (side
  * streams, graph branches), so that one bin's last tasks overlap the next
- * bin's first; 0 runs them one after another on the caller's stream.  The
- * tuning of a new plan (every tile, concurrent and lanes_alt 0) leaves this
- * to the plan: parallel branches, or one launch for small capacities.
+ * bin's first; 0 runs them one after another on the caller's stream.
+ * A new plan has no tuning (every tile, concurrent and lanes_alt 0 are
+ * reported) and chooses by itself: one launch without bins where its capacity
+ * is small, otherwise every tile in parallel branches.  A tuning that is set,
+ * this one too, is run as it stands.
  * Every tuning gives the same (exact) scores; only the time differs. */
 typedef struct {
     uint32_t tiles16;
@@ -114,14 +116,15 @@ int ga_plan_stats(ga_plan *plan, void *stream, ga_stats *stats);
  * and keeps a candidate only when it saves more than 1 %: first dropping
  * every tile that no pair of the sample uses (one launch each; the widest
  * int16x2 tile stays, and the int32 tiles go when the sample has no int32
- * pair; a new plan's bins stay concurrent), then bins one after another vs
- * concurrent, then, greedily,
- * removing one active non-empty tile at a time.  Later batches with pairs
- * in a dropped tile's range run on the next wider active tile (or the
- * intra-sequence kernel), so their scores stay exact.
- * The fastest tuning is kept by the plan and copied to *out (nullable);
- * *ms_best (nullable) gets its median time.  `scores` (device,
- * int32[npairs]) receives the sample's scores. */
+ * pair; a new plan's bins start concurrent; tried in line and concurrent),
+ * then bins one after another vs concurrent, then, greedily, removing one
+ * active non-empty tile at a time.  A new plan of small capacity goes on with
+ * its one launch unless these bins are faster by more than 1 %.  Later
+ * batches with pairs in a dropped tile's range run on the next wider active
+ * tile (or the intra-sequence kernel), so their scores stay exact.
+ * The fastest tuning of the bins is kept by the plan and copied to *out
+ * (nullable); *ms_best (nullable) gets the median time of what the plan
+ * runs.  `scores` (device, int32[npairs]) receives the sample's scores. */
 int ga_plan_autotune(ga_plan *plan, const uint8_t *q_codes, const int64_t *q_off,
                      const uint8_t *t_codes, const int64_t *t_off, int64_t npairs,
                      int32_t *scores, int32_t reps, void *stream, ga_tuning *out,

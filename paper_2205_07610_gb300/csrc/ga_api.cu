@@ -1953,7 +1953,8 @@ struct PlanImpl {
   int occ16[kKaNumBins] = {}, occ32[kKaNumBins] = {}, occ16alt[kKaNumBins] = {};
   int occ_kb = 0, long_grid = 0;
   bool long_packed = false;
-  bool one_launch = false;  // capacity and scoring of the small-batch kernel (used while the tuning is the default)
+  bool one_launch = false;  // capacity and scoring of the small-batch kernel
+  bool tuned = false;       // the plan runs `tune`; until then it chooses by itself
   size_t long_smem = 0;
   Small *small = nullptr;
   int32_t *hist = nullptr, *cursor = nullptr;
@@ -2073,11 +2074,6 @@ int plan_create(const ga_scoring *scoring, int32_t mode, int64_t max_pairs, int6
   return GA_OK;
 }
 
-bool default_tuning(const ga_tuning &t) {
-  const uint32_t all = (1u << kKaNumBins) - 1;
-  return t.tiles16 == all && t.tiles32 == all && t.concurrent == 0 && t.lanes_alt == 0;
-}
-
 // One run, enqueued on s with no host synchronisation and no allocation.
 int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, const uint8_t *t_codes,
                  const int64_t *t_off, int64_t npairs, int32_t *scores, cudaStream_t s) {
@@ -2087,7 +2083,7 @@ int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, cons
   if (cudaGetDevice(&cur) != cudaSuccess || cur != P.dev) return GA_ERR_ARG;
   if (cudaMemsetAsync(P.small, 0, sizeof(Small), s) != cudaSuccess) return GA_ERR_CUDA;
   if (npairs == 0) return GA_OK;
-  if (P.one_launch && default_tuning(P.tune)) {
+  if (P.one_launch && !P.tuned) {
     KRParams kp = make_kr(P.sc, q_codes, q_off, t_codes, t_off, npairs, scores, P.small);
     kp.plan = 1;
     kp.cap = P.max_res;
@@ -2157,12 +2153,12 @@ int plan_enqueue(PlanImpl &P, const uint8_t *q_codes, const int64_t *q_off, cons
   ka.rerun_count = &P.small->rerun_range[1];
 
   // every bin (widest first) plus the long class, one persistent launch
-  // each; concurrent: round-robin over the side streams, joined on s.  An untuned
-  // plan launches every tile, most of them for a few pairs or none, so its bins
+  // each; concurrent: round-robin over the side streams, joined on s.  A plan without
+  // a tuning launches every tile, most of them for a few pairs or none, so its bins
   // run as parallel branches.  GB300, us a replay, in line / parallel: 50,000 pairs
   // of 100..300 1,586 / 543, 50,000 of 150 487 / 377, 20,000 of 300..900 3,942 /
   // 3,282, 1,000 of 400..1,000 670 / 473.
-  const bool conc = P.tune.concurrent != 0 || default_tuning(P.tune);
+  const bool conc = P.tune.concurrent != 0 || !P.tuned;
   int nlaunch = 0, counter = 0;
   auto stream_for = [&](int i) { return conc ? P.side[i % kPlanSide] : s; };
   if (conc) {
@@ -2315,10 +2311,17 @@ int plan_autotune(PlanImpl &P, const uint8_t *qc, const int64_t *qo, const uint8
                   int64_t npairs, int32_t *scores, int reps, cudaStream_t s, ga_tuning *out, float *ms_out) {
   if (reps < 1 || reps > 1000) return GA_ERR_ARG;
   P.drop_graph();
-  ga_tuning best = P.tune;
-  float tbest = 0.f;
-  int rc = plan_time(P, qc, qo, tc, to, npairs, scores, reps, s, &tbest);
+  // What a plan without a tuning runs: the one-launch kernel, a candidate of its own
+  // below, or every tile in parallel branches, from where its bins are tuned.
+  const bool own = !P.tuned && P.one_launch;
+  float tbest = 0.f, town = 0.f;
+  int rc = own ? plan_time(P, qc, qo, tc, to, npairs, scores, reps, s, &town) : GA_OK;
   if (rc) return rc;
+  ga_tuning best = P.tune;
+  if (!P.tuned) best.concurrent = 1;
+  P.tuned = true;
+  P.tune = best;
+  if ((rc = plan_time(P, qc, qo, tc, to, npairs, scores, reps, s, &tbest))) return rc;
   auto consider = [&](ga_tuning cand) -> int {
     P.tune = cand;
     float t = 0.f;
@@ -2356,13 +2359,18 @@ int plan_autotune(PlanImpl &P, const uint8_t *qc, const int64_t *qo, const uint8
     if ((rc = live_mask(0, &l16)) || (rc = live_mask(1, &l32))) return rc;
     if (l16 != best.tiles16 || l32 != best.tiles32) {
       ga_tuning cand = best;
-      if (default_tuning(best)) cand.concurrent = 1;  // as the untuned plan runs
       // keep the widest tile of each class so that the pairs of its range
       // stay on the inter-sequence kernels
       cand.tiles16 = l16 | (best.tiles16 & (1u << (kKaNumBins - 1)));
       cand.tiles32 = l32 | (best.tiles32 & (1u << (kKaNumBins - 1)));
       if (l32 == 0) cand.tiles32 = 0;
-      if ((rc = consider(cand))) return rc;
+      // (both ways: side by side the launches of empty tiles cost little, but the
+      // tiles that are left can be faster one after another)
+      const int32_t given = cand.concurrent;
+      for (const int32_t conc : {given, (int32_t)!given}) {
+        cand.concurrent = conc;
+        if ((rc = consider(cand))) return rc;
+      }
     }
   }
   // 2. bins one after another or concurrent
@@ -2426,6 +2434,10 @@ int plan_autotune(PlanImpl &P, const uint8_t *qc, const int64_t *qo, const uint8
       cand.lanes_alt ^= 1u << b;
       if ((rc = consider(cand))) return rc;
     }
+  }
+  if (own && !(tbest < town * 0.99f)) {
+    tbest = town;
+    P.tuned = false;
   }
   P.tune = best;
   if (out) *out = best;
@@ -2856,6 +2868,7 @@ int ga_plan_set_tuning(ga_plan *plan, const ga_tuning *tuning) {
     return GA_ERR_ARG;
   plan->impl->drop_graph();
   plan->impl->tune = *tuning;
+  plan->impl->tuned = true;
   return GA_OK;
 }
 
