@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(32 * kKrWarps, 4) kr_kernel(const __grid_const
         val = kx_strip<MODE, 8, kFc, false, 1>(v, 0, t, ring, in, ring, nullptr, nullptr, tab, status, KXNoHook{});
       else
         val = kx_strip<MODE, 12, kFc, false, 1>(v, 0, t, ring, in, ring, nullptr, nullptr, tab, status, KXNoHook{});
-      if (t == 0) {
+      if (t == 0 && !status) {  // (as planning counts: pairs without an invalid code)
         atomicAdd(p.cells, (unsigned long long)m * (unsigned long long)n);
         atomicAdd(p.computed, 1);
       }
