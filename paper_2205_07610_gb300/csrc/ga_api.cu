@@ -627,7 +627,7 @@ int kx_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPl
 
 // Launch count, long-class grid and edge buffer of a read-back plan.  The
 // buffer is allocated here, before the fork: the side streams start after it.
-int launch_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPlan &p) {
+int launch_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, ChunkPlan &p, bool strips) {
   p.nlaunch = 0;
   p.counter = 0;
   if (p.npairs == 0) return GA_OK;
@@ -638,7 +638,9 @@ int launch_prepare(Call &c, Alloc &work, const SetView &Q, const SetView &T, Chu
   const bool profile = !c.dna;
   p.long_smem = profile ? (size_t)kKbWarps * (size_t)(c.sc.A + 1) * (32 * kKbK) : 0;
   if (p.long_cnt > 0) {
-    if (int rc = kx_prepare(c, work, Q, T, p)) return rc;
+    p.kx_tile = -1;
+    if (strips)
+      if (int rc = kx_prepare(c, work, Q, T, p)) return rc;
     if (p.kx_tile >= 0) return GA_OK;
     int occ = 0;
     if (long_packed(c.sc, c.dna))
@@ -844,8 +846,19 @@ int run_plans(Call &c, const SetView &Q, const SetView &T, ChunkPlan *ps, int n)
   for (int k = 0; k < n; ++k)
     if ((rc = plan_enqueue(c, Q, T, ps[k]))) return rc;
   if ((rc = plan_readback(c, ps, n))) return rc;
-  for (int k = 0; k < n; ++k)
-    if ((rc = launch_prepare(c, work, Q, T, ps[k]))) return rc;
+  // Where the strips of one plan leave no room for another's edges, all long pairs run
+  // on the kernels that take one warp a pair and the least memory.
+  for (int k = 0, strips = 1; k < n; ++k) {
+    rc = launch_prepare(c, work, Q, T, ps[k], strips);
+    if (rc == GA_ERR_OOM && strips) {
+      work.release();
+      work.failed = strips = false;
+      cudaGetLastError();
+      k = -1;
+    } else if (rc) {
+      return rc;
+    }
+  }
   if ((rc = launch_plans(c, Q, T, ps, n))) return rc;
   for (int k = 0; k < n; ++k)
     if ((rc = rerun_enqueue(c, Q, T, ps[k]))) return rc;
