@@ -929,9 +929,12 @@ struct Events {
 
 // Batches that go to the one-launch kernel first, and plans whose capacity it
 // takes.  Its strips pad a pair to 256, 512 or 768 columns, so it is the slower
-// kernel once the chip is full.  GB300, us a call, planned / one launch: 1,000
-// pairs of 150 residues 183 / 70, 4,000 of 100..300 349 / 164, 8,000 of 250..500
-// 480 / 444, 16,000 of 250..500 682 / 796.  In a plan's graph, where neither waits
+// kernel once the chip is full.  GB300, us a call, local, planned / one launch:
+// 4,000 pairs of 180..200 residues 199 / 130, of 270..300 239 / 206, of 100..500 604 /
+// 230; 8,000 of 180..200 226 / 172, of 340..380 390 / 396, of 384..400 464 / 430, of
+// 100..500 604 / 343, of 270..300 295 / 328: pairs of one length just above a strip's
+// width lose a tenth there, but the lengths are on the device, and reading them first
+// would cost every batch a round trip.  In a plan's graph, where neither waits
 // for the host: 9,000 of 100..300 430 / 217, 16,000 444 / 340, 24,000 466 / 482;
 // 16,000 of 150 186 / 182, 24,000 231 / 260; 16,000 of 250..500 661 / 736.
 constexpr int64_t kKrPairs = 8192;
@@ -2695,7 +2698,7 @@ int ga_align_long(const uint8_t *q, int64_t m, const uint8_t *t, int64_t n, cons
       return GA_ERR_RANGE;
     // every strip of columns on its own warp, about a hundred rows behind its
     // left neighbour (relative int16 cells); other scorings in int32 strips of
-    // 512 columns up to 65536 residues, longer on one warp
+    // 512 columns; pairs beyond 65536 residues are planned as a batch of one
     if (m > 0 && n > 0 && std::max(m, n) <= 65536 && std::max(sc.smax, 0) + sc.alpha <= kKxMaxStep)
       return kx_align_pair(q, m, t, n, sc, mode, score, s, stats);
     if (m <= 65536 && n <= 65536)

@@ -5,10 +5,10 @@
 // Why.  A batch of a thousand reads is 2e7 cells, 2 us of the chip's ALU rate;
 // through the planned path it is a dozen small kernels (packing, validation,
 // keys, a counting sort), three host round trips and one launch per tile width,
-// each with a few warps.  A plan's graph of the same batch holds 40 kernels.  Here nothing is packed or sorted, and the rows of a pair are the latency
-// of a lone strip: 1,000 pairs of 150 x 150 in one call 183 -> 70 us, 1,000 pairs
-// of 100..300 in a plan's graph 553 -> 58 us (GB300, the call and the wait for
-// it).  Larger batches go the planned way, whose tiles pad less and hold two
+// each with a few warps.  A plan's graph of the same batch holds 40 kernels.  Here
+// nothing is packed or sorted, and the rows of a pair are the latency of a lone
+// strip: 1,000 pairs of 150 x 150 in one call 135 -> 58 us, 1,000 pairs of 100..300
+// in a plan's graph 560 -> 44 us (GB300, the call and the wait for it).  Larger batches go the planned way, whose tiles pad less and hold two
 // pairs a lane (the limits stand beside the two callers).
 //
 // Strips of 256, 512 or 768 columns (K = 4, 8, 12) by the longer sequence, with

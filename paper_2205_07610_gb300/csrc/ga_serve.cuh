@@ -85,7 +85,7 @@ struct SvScoring {
 struct SvRequest {
   const uint8_t *q;     // device codes
   const uint8_t *t;
-  int2 *edges;          // (nstrips - 1) edges of R + 1 int2 each
+  int2 *edges;          // int32 strips: (nstrips - 1) edges of R + 1 int2; packed ones share R + 1 words
   int32_t *out;         // nullable: the score is also stored here
   int64_t id;
   int32_t m, n;
