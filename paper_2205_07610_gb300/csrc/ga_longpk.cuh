@@ -374,9 +374,11 @@ __global__ void __launch_bounds__(128, MODE == kModeSemi ? 3 : 0) kw_kernel(cons
             H[j] = __vadd2(H[j], dl);
             E[j] = __vadd2(E[j], dl);
           }
-          Hdiag = __vadd2(Hdiag, dl);
-          Hleft = __vadd2(Hleft, dl);
-          Fin = __vadd2(Fin, dl);
+          // (the left inputs can be -inf, past the last row of the left edge)
+          const uint32_t dp = pk16(d0, d1);
+          Hdiag = __vmaxs2(__vsubss2(Hdiag, dp), NEGV);
+          Hleft = __vmaxs2(__vsubss2(Hleft, dp), NEGV);
+          Fin = __vmaxs2(__vsubss2(Fin, dp), NEGV);
           if constexpr (MODE == kModeLocal) {  // the zero of Eq. H under the new bases
             Z = pk16(::max(-b[0], kNeg16), ::max(-b[1], kNeg16));
 #pragma unroll
